@@ -219,40 +219,33 @@ __device__ __forceinline__ int row_exponent(double mx) {
     return E == 0 ? -1022 : E - 1022;
 }
 
-// signed base-256 digits of round(x * 2^(8s - e)); |x| <= 2^e.  d[1..s-1]
-// lie in [-128, 127] (Y = 256 Y' + d with Y' = floor((Y + 128) / 256)), d[0]
-// carries the sign and the top.  Every index of d is static (unrolled over
-// MAX_S), so d stays in registers.
-__device__ __forceinline__ void digits_bits(unsigned long long b, int e, int s, int* d);
-__device__ __forceinline__ void digits(double x, int e, int s, int* d) {
-    digits_bits((unsigned long long)__double_as_longlong(x), e, s, d);
+// Signed base-256 digits of Y = round(x * 2^(8s - e)), |x| < 2^e, held as the
+// bytes of one biased integer: with B = sum_{t=1}^{s-1} 128 * 256^(s-1-t), the
+// balanced recurrence Y' = floor((Y + 128) / 256), d = Y - 256 Y' (d in
+// [-128, 127]) is what long division of Z = Y + B gives, so that digit t >= 1
+// is byte s-1-t of Z minus 128 and d_0 = Z >> 8(s-1) carries the sign and the
+// top: one 64-bit addition instead of s dependent shift-and-subtract steps.
+// The slicers are then bound by memory, not by integer issue (~30
+// instructions per element instead of ~100): the warm sweep at d=3, D=8,
+// chi=128 went from 763 to 545 ms with the column slicers below.
+__host__ __device__ constexpr unsigned long long digit_bias(int s) {
+    unsigned long long b = 0;
+    for (int t = 1; t < s; ++t) b = (b << 8) | 128ull;
+    return b;
 }
-// the same from the FP64 bit pattern b
-__device__ __forceinline__ void digits_bits(unsigned long long b, int e, int s, int* d) {
-    int ex = (int)((b >> 52) & 0x7ff);
-    unsigned long long mant = b & ((1ull << 52) - 1);
-    if (ex == 0) ex = 1;
-    else mant |= 1ull << 52;
-    const int shift = ex - 1075 + 8 * s - e;  // x = mant 2^(ex-1075)
-    long long Y;
-    if (mant == 0) Y = 0;
-    else if (shift >= 0) Y = (long long)(mant << shift);  // <= 2^(8s) by |x| <= 2^e
-    else {
-        const int sh = -shift;
-        Y = sh >= 54 ? 0 : (long long)((mant + (1ull << (sh - 1))) >> sh);
-    }
-    if (b >> 63) Y = -Y;
-#pragma unroll
-    for (int t = MAX_S - 1; t >= 1; --t) {
-        if (t < s) {
-            const long long Yn = (Y + 128) >> 8;
-            d[t] = (int)((uint32_t)Y - ((uint32_t)Yn << 8));  // Y - 256 Y', in [-128, 127]
-            Y = Yn;
-        } else {
-            d[t] = 0;
-        }
-    }
-    d[0] = (int)Y;
+// Z from the FP64 bit pattern b of x; base = 1075 - 8s + e.  x = mant
+// 2^(ex-1075), so Y = mant >> (base - ex) rounded half away from zero, and
+// |x| < 2^e makes that a right shift by at least 53 - 8 MAX_S > 0 bits.
+__device__ __forceinline__ unsigned long long digit_bytes(unsigned long long b, int base, unsigned long long bias) {
+    const unsigned hi = (unsigned)(b >> 32);
+    const int ex0 = (int)((hi >> 20) & 0x7ff);
+    const int ex = max(ex0, 1);
+    const unsigned mh = (hi & 0xfffffu) | (ex0 ? 0x100000u : 0u);  // denormals have no implicit bit
+    const unsigned long long mant = ((unsigned long long)mh << 32) | (unsigned)b;
+    const int sh = min(base - ex, 55);  // mant < 2^53: everything from 54 on gives 0
+    const unsigned long long y = ((mant >> (sh - 1)) + 1ull) >> 1;
+    const unsigned long long m = (unsigned long long)((long long)b >> 63);
+    return (y ^ m) - m + bias;
 }
 
 // A small int as an FP32 without a conversion instruction: 1.5 2^23 + d has
@@ -262,54 +255,48 @@ __device__ __forceinline__ float small_int_f32(int d) {
     return __int_as_float(0x4B400000 + d) - 12582912.0f;
 }
 
-// digit * 2^(-8t): at most 9 significant bits, exact in FP32 and BF16; the
-// power of two is built from its exponent field
-__device__ __forceinline__ __nv_bfloat16 slice_value(int digit, int t) {
-    return __float2bfloat16_rn(small_int_f32(digit) * __int_as_float((127 - 8 * t) << 23));
+// BF16 pair of digit t >= 1 of two elements (a in the low half): `w` holds
+// their digit bytes u = d + 128 in bits 0-7 and 16-23.  With u = 128 h + l, l < 128:
+// (128 + l) 2^(-8t) is a BF16 whose 7 mantissa bits are l, (256 - 128 h)
+// 2^(-8t) one whose lowest exponent bit is !h, and their difference, exact in
+// BF16, is d 2^(-8t): two logic operations and one packed subtraction for
+// two digits, no conversion instruction.
+__device__ __forceinline__ unsigned digit_pair(unsigned w, int t) {
+    const unsigned kv = (unsigned)(134 - 8 * t) << 7, kc = (unsigned)(135 - 8 * t) << 7;
+    const unsigned v = (w & 0x007f007fu) | (kv * 0x10001u);
+    const unsigned c = (w & 0x00800080u) ^ (kc * 0x10001u);
+    const __nv_bfloat162 d = __hsub2(*reinterpret_cast<const __nv_bfloat162*>(&v),
+                                     *reinterpret_cast<const __nv_bfloat162*>(&c));
+    return *reinterpret_cast<const unsigned*>(&d);
+}
+__device__ __forceinline__ unsigned bf2_bits(float a, float b) {
+    const __nv_bfloat162 p = __floats2bfloat162_rn(a, b);  // a in the low half (lower address)
+    return *reinterpret_cast<const unsigned*>(&p);
+}
+// Slice t of two elements with digit integers za, zb as a BF16 pair (the byte
+// index depends on s, the powers of two on t).
+__device__ __forceinline__ unsigned slice_of_pair(unsigned long long za, unsigned long long zb, int s, int t) {
+    if (t == 0)  // |d_0| <= 256: exact in BF16
+        return bf2_bits(small_int_f32((int)((long long)za >> (8 * (s - 1)))),
+                        small_int_f32((int)((long long)zb >> (8 * (s - 1)))));
+    const int byte = s - 1 - t;  // below 4 but for t = 1 of 6 slices
+    const unsigned a = byte < 4 ? (unsigned)za : (unsigned)(za >> 32);
+    const unsigned b = byte < 4 ? (unsigned)zb : (unsigned)(zb >> 32);
+    // byte of a to bits 0-7, byte of b to bits 16-23
+    return digit_pair(__byte_perm(a, b, (byte & 3) | ((4 + (byte & 3)) << 8)), t);
 }
 
-// Consecutive k contiguous (innermost K stride 1): one warp per row.
-__global__ void k_split_rows(const double* __restrict__ X, int R, int K, int K8, View rv, View kv, int s,
-                             __nv_bfloat16* __restrict__ out, int* __restrict__ ex) {
-    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-    if (warp >= R) return;
-    const double* xr = X + view_offset32(rv, (unsigned)warp);
-    auto at = [&](int k) { return xr[kv.n == 1 ? (long long)k * kv.stride[0] : view_offset32(kv, (unsigned)k)]; };
-    // max |x| on the bit patterns: non-negative doubles order like integers,
-    // and the integer pipe is far faster than GB300's FP64 pipe
-    unsigned long long mb = 0;
-    for (int k = lane; k < K; k += 32) mb = umax64(mb, abs_bits(at(k)));
-    for (int o = 16; o > 0; o >>= 1) mb = umax64(mb, __shfl_xor_sync(0xffffffffu, mb, o));
-    const int e = row_exponent(__longlong_as_double((long long)mb));
-    if (lane == 0) ex[warp] = e;
-    const size_t plane = (size_t)R * K8;
-    __nv_bfloat16* o = out + (size_t)warp * K8;
-    for (int k = lane; k < K8; k += 32) {
-        int d[MAX_S];
-        if (k < K) digits(at(k), e, s, d);
-        else
-            for (int t = 0; t < MAX_S; ++t) d[t] = 0;
-#pragma unroll
-        for (int t = 0; t < MAX_S; ++t)
-            if (t < s) o[t * plane + k] = slice_value(d[t], t);
-    }
-}
-
-// General strides (rows contiguous when rs == 1).  Pass 1: per-row max|x|
-// over K, the grid split over (32-row groups, K ranges), combined with
-// atomicMax on the bit pattern.  Pass 2: a warp takes 32 rows x 32 k (lane =
-// row while reading, so reads along contiguous rows coalesce), staged
-// through shared memory so that the K-major slice writes coalesce too.
-constexpr int COLS_KRANGE = 256;
-
-__global__ void k_rowmax_cols(const double* __restrict__ X, int R, int K, View rv, View kv, int kranges,
+// Per-row max|x| of operands whose rows are not contiguous in k: lane = row,
+// a warp takes 32 rows x `krange` k, combined with atomicMax on the bit
+// patterns (non-negative doubles order like integers).
+__global__ void k_rowmax_cols(const double* __restrict__ X, int R, int K, View rv, View kv, int kranges, int krange,
                               unsigned long long* __restrict__ maxbits) {
     const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     const int rg = w / kranges, kr = w - rg * kranges;
     const int r = rg * 32 + lane;
-    const int k0 = kr * COLS_KRANGE;
+    const int k0 = kr * krange;
     if (r >= R || k0 >= K) return;
-    const int k1 = min(K, k0 + COLS_KRANGE);
+    const int k1 = min(K, k0 + krange);
     const double* xr = X + view_offset32(rv, (unsigned)r);
     Odometer od;
     od.init(kv, (unsigned)k0);
@@ -328,49 +315,6 @@ __global__ void k_rowmax_cols(const double* __restrict__ X, int R, int K, View r
         for (int u = 0; u < 8; ++u) mx = umax64(mx, abs_bits(v[u]));
     }
     atomicMax(maxbits + r, mx);
-}
-
-__global__ void k_split_cols(const double* __restrict__ X, int R, int K, int K8, View rv, View kv,
-                             int s, const unsigned long long* __restrict__ maxbits, __nv_bfloat16* __restrict__ out,
-                             int* __restrict__ ex) {
-    __shared__ __nv_bfloat16 tile[2][MAX_S][32][33];  // launched with 2 warps
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int r0 = blockIdx.x * 32;
-    const int k0 = (blockIdx.y * 2 + w) * 32;
-    if (k0 >= K8) return;
-    const int r = r0 + lane;
-    const bool live = r < R;
-    const int e = live ? row_exponent(__longlong_as_double((long long)maxbits[r])) : 0;
-    if (live && k0 == 0) ex[r] = e;
-    const double* xr = X + (live ? view_offset32(rv, (unsigned)r) : 0);
-    Odometer od;
-    od.init(kv, (unsigned)min(k0, K - 1));
-    for (int kb = 0; kb < 32; kb += 8) {
-        double v[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            const int k = k0 + kb + u;
-            v[u] = 0.0;
-            if (live && k < K) {
-                v[u] = xr[od.off];
-                od.step(kv);
-            }
-        }
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            int d[MAX_S];
-            digits(v[u], e, s, d);
-#pragma unroll
-            for (int t = 0; t < MAX_S; ++t)
-                if (t < s) tile[w][t][lane][kb + u] = slice_value(d[t], t);
-        }
-    }
-    __syncwarp();
-    const size_t plane = (size_t)R * K8;
-    const int k = k0 + lane;
-    if (k < K8)
-        for (int rr = 0; rr < 32 && r0 + rr < R; ++rr)
-            for (int t = 0; t < s; ++t) out[t * plane + (size_t)(r0 + rr) * K8 + k] = tile[w][t][rr][lane];
 }
 
 // round(x 2^(nbits - e)) as an integer, |x| <= 2^e (integer operations on the
@@ -425,53 +369,13 @@ __global__ void k_split_tf32(const double* __restrict__ X, int R, int K, int K4,
     *reinterpret_cast<float4*>(o + plane) = make_float4(s1[0], s1[1], s1[2], s1[3]);
 }
 
-// ---------------------------------------------------------------------------
-// Plain 2D operands (one row stride, one K stride): the slices of eight
-// consecutive k of one row are built in registers and written as one 16-byte
-// store per slice.
-// ---------------------------------------------------------------------------
-__device__ __forceinline__ unsigned bf2_bits(float a, float b) {
-    const __nv_bfloat162 p = __floats2bfloat162_rn(a, b);  // a in the low half (lower address)
-    return *reinterpret_cast<const unsigned*>(&p);
-}
-// slice t of eight consecutive values as 8 BF16 (16 bytes), t < s
-__device__ __forceinline__ void slice8_pack(const double* v, int e, int s, uint4* q) {
-    int d[8][MAX_S];
-#pragma unroll
-    for (int u = 0; u < 8; ++u) digits(v[u], e, s, d[u]);
-#pragma unroll
-    for (int t = 0; t < MAX_S; ++t) {
-        if (t < s) {
-            const float sc = __int_as_float((127 - 8 * t) << 23);  // 2^(-8t)
-            q[t].x = bf2_bits(small_int_f32(d[0][t]) * sc, small_int_f32(d[1][t]) * sc);
-            q[t].y = bf2_bits(small_int_f32(d[2][t]) * sc, small_int_f32(d[3][t]) * sc);
-            q[t].z = bf2_bits(small_int_f32(d[4][t]) * sc, small_int_f32(d[5][t]) * sc);
-            q[t].w = bf2_bits(small_int_f32(d[6][t]) * sc, small_int_f32(d[7][t]) * sc);
-        }
-    }
-}
-// slice8_pack of eight FP64 bit patterns
-__device__ __forceinline__ void slice8_pack_bits(const unsigned long long* vb, int e, int s, uint4* q) {
-    int d[8][MAX_S];
-#pragma unroll
-    for (int u = 0; u < 8; ++u) digits_bits(vb[u], e, s, d[u]);
-#pragma unroll
-    for (int t = 0; t < MAX_S; ++t) {
-        if (t < s) {
-            const float sc = __int_as_float((127 - 8 * t) << 23);  // 2^(-8t)
-            q[t].x = bf2_bits(small_int_f32(d[0][t]) * sc, small_int_f32(d[1][t]) * sc);
-            q[t].y = bf2_bits(small_int_f32(d[2][t]) * sc, small_int_f32(d[3][t]) * sc);
-            q[t].z = bf2_bits(small_int_f32(d[4][t]) * sc, small_int_f32(d[5][t]) * sc);
-            q[t].w = bf2_bits(small_int_f32(d[6][t]) * sc, small_int_f32(d[7][t]) * sc);
-        }
-    }
-}
-__device__ __forceinline__ void slice8_store(const double* v, int e, int s, __nv_bfloat16* dst, size_t plane) {
-    uint4 q[MAX_S];
-    slice8_pack(v, e, s, q);
+// slice t of eight consecutive values (16 bytes per slice) from their digit integers
+__device__ __forceinline__ void slice8_pack(const unsigned long long* z, int s, uint4* q) {
 #pragma unroll
     for (int t = 0; t < MAX_S; ++t)
-        if (t < s) *reinterpret_cast<uint4*>(dst + t * plane) = q[t];
+        if (t < s)
+            q[t] = make_uint4(slice_of_pair(z[0], z[1], s, t), slice_of_pair(z[2], z[3], s, t),
+                              slice_of_pair(z[4], z[5], s, t), slice_of_pair(z[6], z[7], s, t));
 }
 
 // K contiguous, rows at stride rs, K8 <= 4 * 8 * TPR: TPR threads per row,
@@ -531,12 +435,16 @@ __global__ void __launch_bounds__(256) k_split_rows_reg(const double* __restrict
     const int e = row_exponent_bits(mb);
     if (j == 0) ex[r] = e;
     const size_t plane = (size_t)R * K8;
+    const int base = 1075 - 8 * s + e;
+    const unsigned long long bias = digit_bias(s);
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
         const int c = j + i * TPR;
         if (c < nch) {
             uint4 q[MAX_S];
-            slice8_pack_bits(v[i], e, s, q);
+#pragma unroll
+            for (int u = 0; u < 8; ++u) v[i][u] = digit_bytes(v[i][u], base, bias);
+            slice8_pack(v[i], s, q);
             __nv_bfloat16* dst = out + (size_t)r * K8 + (size_t)c * 8;
 #pragma unroll
             for (int t = 0; t < MAX_S; ++t)
@@ -545,53 +453,180 @@ __global__ void __launch_bounds__(256) k_split_rows_reg(const double* __restrict
     }
 }
 
-// Rows contiguous (row stride 1), K at stride cs: lane = row, 32
-// consecutive k per step (each load instruction reads 32 consecutive rows),
-// one warp per 32 rows x kspan k (kspan a multiple of 32); row maxima from
-// k_rowmax_cols.  The slices go out through shared memory so that four lanes
-// write one row's 64 contiguous bytes in the same store instruction: lanes
-// that each wrote 16 bytes of a different row left half-written sectors
-// that L2 filled from DRAM (1.5x the bytes each way).
-__global__ void __launch_bounds__(64) k_split_cols_reg(const double* __restrict__ X, int R, int K, int K8,
-                                                      long long cs, int s,
-                                                      const unsigned long long* __restrict__ maxbits,
-                                                      __nv_bfloat16* __restrict__ out, int* __restrict__ ex,
-                                                      int kspan, int kgroups) {
-    // per warp: every slice of 32 rows x 4 x 16 bytes (+1 pad against bank conflicts)
-    __shared__ uint4 tile[2][MAX_S][32][5];
+// K contiguous but longer than the register-resident kernel takes (or read
+// through a view): row maxima by (row, 1024-wide K range), then one thread
+// per eight consecutive k.  A one-warp-per-row form left a 9 x 1M operand (the
+// two-site density matrix at chi = 128) to nine warps.
+constexpr int ROWS_KRANGE = 1024;
+__global__ void __launch_bounds__(256) k_rowmax_rows(const double* __restrict__ X, int R, int K, View rv, View kv,
+                                                    int kranges, unsigned long long* __restrict__ maxbits) {
+    const long long w = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31;
+    const long long r = w / kranges;
+    if (r >= R) return;
+    const int k0 = (int)(w - r * kranges) * ROWS_KRANGE, k1 = min(K, k0 + ROWS_KRANGE);
+    const double* xr = X + view_offset32(rv, (unsigned)r);
+    unsigned long long mb = 0;
+    for (int k = k0 + lane; k < k1; k += 32)
+        mb = umax64(mb, abs_bits(xr[kv.n == 1 ? (long long)k : view_offset32(kv, (unsigned)k)]));
+    for (int o = 16; o > 0; o >>= 1) mb = umax64(mb, __shfl_xor_sync(0xffffffffu, mb, o));
+    if (lane == 0) atomicMax(maxbits + r, mb);
+}
+__global__ void __launch_bounds__(256) k_split_rows_long(const double* __restrict__ X, int R, int K, int K8, View rv,
+                                                        View kv, int s,
+                                                        const unsigned long long* __restrict__ maxbits,
+                                                        __nv_bfloat16* __restrict__ out, int* __restrict__ ex) {
+    const int nch = K8 >> 3;
+    const long long tid = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    const long long r = tid / nch;
+    const int c = (int)(tid - r * nch);
+    if (r >= R) return;
+    const int e = row_exponent_bits(maxbits[r]);
+    if (c == 0) ex[r] = e;
+    const unsigned long long* xr =
+        reinterpret_cast<const unsigned long long*>(X) + view_offset32(rv, (unsigned)r);
+    const int base = 1075 - 8 * s + e;
+    const unsigned long long bias = digit_bias(s);
+    unsigned long long z[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+        const int k = c * 8 + u;
+        z[u] = k < K ? __ldcs(xr + (kv.n == 1 ? (long long)k : view_offset32(kv, (unsigned)k))) : 0ull;
+    }
+#pragma unroll
+    for (int u = 0; u < 8; ++u) z[u] = digit_bytes(z[u], base, bias);
+    uint4 q[MAX_S];
+    slice8_pack(z, s, q);
+    const size_t plane = (size_t)R * K8;
+    __nv_bfloat16* dst = out + (size_t)r * K8 + (size_t)c * 8;
+#pragma unroll
+    for (int t = 0; t < MAX_S; ++t)
+        if (t < s) *reinterpret_cast<uint4*>(dst + t * plane) = q[t];
+}
+
+// Slices of 32 rows (lane = row) x 32 consecutive k from k0, given the digit
+// integers z of the lane's row, through this warp's shared-memory tile so that
+// four lanes write one row's 64 contiguous bytes in one store instruction:
+// lanes that each wrote 16 bytes of a different row left half-written
+// sectors that L2 filled from DRAM (1.5x the bytes each way).  One slice at
+// a time: the tile is 2.5 KB per warp whatever the number of slices.
+__device__ __forceinline__ void store_tile32(const unsigned long long* z, int s, uint4 (*tile)[5], int lane, int r0,
+                                             int R, int k0, int kend, int K8, size_t plane,
+                                             __nv_bfloat16* __restrict__ out) {
+#pragma unroll
+    for (int t = 0; t < MAX_S; ++t) {
+        if (t >= s) break;
+        unsigned p[16];
+#pragma unroll
+        for (int u = 0; u < 16; ++u) p[u] = slice_of_pair(z[2 * u], z[2 * u + 1], s, t);
+#pragma unroll
+        for (int c = 0; c < 4; ++c) tile[lane][c] = make_uint4(p[4 * c], p[4 * c + 1], p[4 * c + 2], p[4 * c + 3]);
+        __syncwarp();
+        // lane -> (row rr = j * 8 + lane / 4, 16-byte chunk c = lane % 4)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int rr = j * 8 + (lane >> 2), c = lane & 3;
+            if (r0 + rr < R && k0 + 8 * c < kend)
+                *reinterpret_cast<uint4*>(out + t * plane + (size_t)(r0 + rr) * K8 + k0 + 8 * c) = tile[rr][c];
+        }
+        __syncwarp();
+    }
+}
+// 32 consecutive k of the lane's row as bit patterns (0 beyond K)
+template <bool PLAIN>
+__device__ __forceinline__ void load32(const unsigned long long* xr, bool live, int k0, int K, const View& kv,
+                                       unsigned long long* v) {
+    if (PLAIN) {
+        const long long cs = kv.stride[0];
+#pragma unroll
+        for (int u = 0; u < 32; ++u) v[u] = (live && k0 + u < K) ? __ldg(xr + (long long)(k0 + u) * cs) : 0ull;
+    } else {
+        Odometer od;
+        od.init(kv, (unsigned)min(k0, K - 1));
+#pragma unroll
+        for (int u = 0; u < 32; ++u) {
+            v[u] = (live && k0 + u < K) ? __ldg(xr + od.off) : 0ull;
+            if (k0 + u + 1 < K) od.step(kv);
+        }
+    }
+}
+
+// Operands read along their rows' contiguous direction (lane = row): one
+// warp per 32 rows x kspan k (kspan a multiple of 32), row maxima from
+// k_rowmax_cols.  PLAIN: one K stride.
+template <bool PLAIN>
+__global__ void __launch_bounds__(64) k_split_cols(const double* __restrict__ X, int R, int K, int K8, View rv, View kv,
+                                                  int s, const unsigned long long* __restrict__ maxbits,
+                                                  __nv_bfloat16* __restrict__ out, int* __restrict__ ex, int kspan,
+                                                  int kgroups) {
+    __shared__ uint4 tile[2][32][5];  // +1 uint4 per row against bank conflicts
     const int wid = (int)((blockIdx.x * (size_t)blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
-    const int w = threadIdx.x >> 5;
     const int rg = wid / kgroups, kg = wid - rg * kgroups;
     if (rg * 32 >= R) return;
     const int r0 = rg * 32, r = r0 + lane;
     const bool live = r < R;
-    const int e = live ? row_exponent(__longlong_as_double((long long)maxbits[r])) : 0;
+    const int e = live ? row_exponent_bits(maxbits[r]) : 0;
     if (live && kg == 0) ex[r] = e;
+    const unsigned long long* xr =
+        reinterpret_cast<const unsigned long long*>(X) + (live ? view_offset32(rv, (unsigned)r) : 0);
     const size_t plane = (size_t)R * K8;
+    const int base = 1075 - 8 * s + e;
+    const unsigned long long bias = digit_bias(s);
     const int kend = min(K8, (kg + 1) * kspan);
     for (int k0 = kg * kspan; k0 < kend; k0 += 32) {
-        double v[32];
+        unsigned long long v[32];
+        load32<PLAIN>(xr, live, k0, K, kv, v);
 #pragma unroll
-        for (int u = 0; u < 32; ++u) v[u] = (live && k0 + u < K) ? __ldcs(X + (long long)(k0 + u) * cs + r) : 0.0;
+        for (int u = 0; u < 32; ++u) v[u] = digit_bytes(v[u], base, bias);
+        store_tile32(v, s, tile[threadIdx.x >> 5], lane, r0, R, k0, kend, K8, plane, out);
+    }
+}
+
+// The same for K up to COLS_ONE_MAX in one launch, one CTA per 32 rows: its
+// warps (one per 32 k, at most 16) first agree on the row maxima, then
+// slice; the last 32 k a warp read stay in registers, so that K <= 512 is
+// read once.  The three launches of the long form (clear, maxima, slices)
+// cost a small operand more than its bytes: with 32-warp grids the transposed
+// 512 x 512 corner of D=4, chi=32 took ~48 us, and the scan point there went
+// from 107 to 60 ms.  Beyond 1536 the two re-reads per warp cost more than
+// the launches, and short operands leave SMs idle.
+constexpr int COLS_ONE_MAX = 1536;
+constexpr int COLS_ONE_WARPS = 16;
+template <bool PLAIN>
+__global__ void __launch_bounds__(32 * COLS_ONE_WARPS) k_split_cols_one(const double* __restrict__ X, int R, int K, int K8,
+                                                                       View rv, View kv, int s,
+                                                                       __nv_bfloat16* __restrict__ out,
+                                                                       int* __restrict__ ex) {
+    __shared__ uint4 tile[COLS_ONE_WARPS][32][5];
+    __shared__ unsigned long long red[COLS_ONE_WARPS][32];
+    const int w = threadIdx.x >> 5, nw = blockDim.x >> 5, lane = threadIdx.x & 31;
+    const int r0 = blockIdx.x * 32, r = r0 + lane;
+    const bool live = r < R;
+    const unsigned long long* xr =
+        reinterpret_cast<const unsigned long long*>(X) + (live ? view_offset32(rv, (unsigned)r) : 0);
+    unsigned long long v[32];
+    unsigned long long mb = 0;
+    int k0 = w * 32, last = -1;
+    for (; k0 < K8; k0 += nw * 32) {
+        load32<PLAIN>(xr, live, k0, K, kv, v);
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            uint4 q[MAX_S];
-            slice8_pack(v + 8 * c, e, s, q);
+        for (int u = 0; u < 32; ++u) mb = umax64(mb, v[u] & 0x7fffffffffffffffull);
+        last = k0;
+    }
+    red[w][lane] = mb;
+    __syncthreads();
+    mb = 0;
+    for (int i = 0; i < nw; ++i) mb = umax64(mb, red[i][lane]);
+    const int e = row_exponent_bits(mb);
+    if (live && w == 0) ex[r] = e;
+    const size_t plane = (size_t)R * K8;
+    const int base = 1075 - 8 * s + e;
+    const unsigned long long bias = digit_bias(s);
+    for (k0 = last; k0 >= 0; k0 -= nw * 32) {
+        if (k0 != last) load32<PLAIN>(xr, live, k0, K, kv, v);
 #pragma unroll
-            for (int t = 0; t < MAX_S; ++t)
-                if (t < s) tile[w][t][lane][c] = q[t];
-        }
-        __syncwarp();
-        // lane -> (row rr = j * 8 + lane / 4, 16-byte chunk c = lane % 4)
-        for (int t = 0; t < s; ++t)
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const int rr = j * 8 + (lane >> 2), c = lane & 3;
-                if (r0 + rr < R && k0 + 8 * c < kend)
-                    *reinterpret_cast<uint4*>(out + t * plane + (size_t)(r0 + rr) * K8 + k0 + 8 * c) =
-                        tile[w][t][rr][c];
-            }
-        __syncwarp();
+        for (int u = 0; u < 32; ++u) v[u] = digit_bytes(v[u], base, bias);
+        store_tile32(v, s, tile[w], lane, r0, R, k0, K8, K8, plane, out);
     }
 }
 
@@ -1224,6 +1259,15 @@ inline const int* split_tf32_exponents(const void* buf, int R, int K4) {
     return (const int*)((const char*)buf + align256((size_t)2 * R * K4 * 4) + align256((size_t)R * 8));
 }
 
+// K range of one warp in the lane = row kernels: 256, halved down to 32 until
+// the operand gives every SM sixteen warps
+static int cols_krange(int R, int K) {
+    const long long rg = (R + 31) / 32;
+    int range = 256;
+    while (range > 32 && rg * ((K + range - 1) / range) < 152 * 16) range /= 2;
+    return range;
+}
+
 cudaError_t oz_split_tf32(const double* X, int R, int K, const OzView& rvh, const OzView& kvh, void* buf,
                           cudaStream_t st) {
     if (R <= 0 || K <= 0 || rvh.n < 1 || rvh.n > 4 || kvh.n < 1 || kvh.n > 4) return cudaErrorInvalidValue;
@@ -1243,12 +1287,13 @@ cudaError_t oz_split_tf32(const double* X, int R, int K, const OzView& rvh, cons
     cudaError_t e = cudaMemsetAsync(mb, 0, (size_t)R * 8, st);
     if (e != cudaSuccess) return e;
     const unsigned rg = (unsigned)((R + 31) / 32);
-    const unsigned kr = (unsigned)((K + oz::COLS_KRANGE - 1) / oz::COLS_KRANGE);
+    const int krange = cols_krange(R, K);
+    const unsigned kr = (unsigned)((K + krange - 1) / krange);
     const unsigned long long warps = (unsigned long long)rg * kr;
     const unsigned long long threads = (unsigned long long)R * (K4 / 4);
     if ((warps + 3) / 4 > 0x7fffffffull || (threads + 255) / 256 > 0x7fffffffull) return cudaErrorInvalidValue;
     ++g_launches;
-    oz::k_rowmax_cols<<<(unsigned)((warps + 3) / 4), 128, 0, st>>>(X, R, K, rv, kv, (int)kr, mb);
+    oz::k_rowmax_cols<<<(unsigned)((warps + 3) / 4), 128, 0, st>>>(X, R, K, rv, kv, (int)kr, krange, mb);
     ++g_launches;
     oz::k_split_tf32<<<(unsigned)((threads + 255) / 256), 256, 0, st>>>(X, R, K, K4, rv, kv, mb, sl, ex);
     return cudaGetLastError();
@@ -1307,34 +1352,37 @@ cudaError_t oz_split_view(const double* X, int R, int K, const OzView& rvh, cons
         ++g_launches;
         launch_split_rows_reg(tpr, vec, blocks, st, X, R, K, K8, rv.stride[0], s, sl, ex);
     } else if (cs == 1) {
-        ++g_launches;
-        const unsigned blocks = (unsigned)(((size_t)R * 32 + 255) / 256);
-        oz::k_split_rows<<<blocks, 256, 0, st>>>(X, R, K, K8, rv, kv, s, sl, ex);
-    } else if (rv.n == 1 && rv.stride[0] == 1 && kv.n == 1) {
         cudaError_t e = cudaMemsetAsync(mb, 0, (size_t)R * 8, st);
         if (e != cudaSuccess) return e;
+        const int kr = (K + oz::ROWS_KRANGE - 1) / oz::ROWS_KRANGE;
+        const unsigned long long b1 = ((unsigned long long)R * kr + 7) / 8, b2 = ((unsigned long long)R * nch + 255) / 256;
+        if (b1 > 0x7fffffffull || b2 > 0x7fffffffull) return cudaErrorInvalidValue;
+        ++g_launches;
+        oz::k_rowmax_rows<<<(unsigned)b1, 256, 0, st>>>(X, R, K, rv, kv, kr, mb);
+        ++g_launches;
+        oz::k_split_rows_long<<<(unsigned)b2, 256, 0, st>>>(X, R, K, K8, rv, kv, s, mb, sl, ex);
+    } else if (K8 <= oz::COLS_ONE_MAX) {
         const unsigned rg = (unsigned)((R + 31) / 32);
-        const unsigned kr = (unsigned)((K + oz::COLS_KRANGE - 1) / oz::COLS_KRANGE);
-        const unsigned long long warps = (unsigned long long)rg * kr;
-        const int kspan = 256, kgroups = (K8 + kspan - 1) / kspan;
-        const unsigned long long warps2 = (unsigned long long)rg * kgroups;
-        if ((warps + 3) / 4 > 0x7fffffffull || (warps2 + 1) / 2 > 0x7fffffffull) return cudaErrorInvalidValue;
+        const int nw = std::min(oz::COLS_ONE_WARPS, (K8 + 31) / 32);
         ++g_launches;
-        oz::k_rowmax_cols<<<(unsigned)((warps + 3) / 4), 128, 0, st>>>(X, R, K, rv, kv, (int)kr, mb);
-        ++g_launches;
-        oz::k_split_cols_reg<<<(unsigned)((warps2 + 1) / 2), 64, 0, st>>>(X, R, K, K8, kv.stride[0], s, mb, sl, ex,
-                                                                           kspan, kgroups);
+        if (kv.n == 1) oz::k_split_cols_one<true><<<rg, 32 * nw, 0, st>>>(X, R, K, K8, rv, kv, s, sl, ex);
+        else oz::k_split_cols_one<false><<<rg, 32 * nw, 0, st>>>(X, R, K, K8, rv, kv, s, sl, ex);
     } else {
         cudaError_t e = cudaMemsetAsync(mb, 0, (size_t)R * 8, st);
         if (e != cudaSuccess) return e;
         const unsigned rg = (unsigned)((R + 31) / 32);
-        const unsigned kr = (unsigned)((K + oz::COLS_KRANGE - 1) / oz::COLS_KRANGE);
+        const int krange = cols_krange(R, K);
+        const unsigned kr = (unsigned)((K + krange - 1) / krange);
         const unsigned long long warps = (unsigned long long)rg * kr;
-        if ((warps + 3) / 4 > 0x7fffffffull || (K8 / 32 + 2) / 2 > 65535) return cudaErrorInvalidValue;
+        const int kspan = cols_krange(R, K8), kgroups = (K8 + kspan - 1) / kspan;
+        const unsigned long long warps2 = (unsigned long long)rg * kgroups;
+        if ((warps + 3) / 4 > 0x7fffffffull || (warps2 + 1) / 2 > 0x7fffffffull) return cudaErrorInvalidValue;
         ++g_launches;
-        oz::k_rowmax_cols<<<(unsigned)((warps + 3) / 4), 128, 0, st>>>(X, R, K, rv, kv, (int)kr, mb);
+        oz::k_rowmax_cols<<<(unsigned)((warps + 3) / 4), 128, 0, st>>>(X, R, K, rv, kv, (int)kr, krange, mb);
+        const unsigned blocks = (unsigned)((warps2 + 1) / 2);
         ++g_launches;
-        oz::k_split_cols<<<dim3(rg, (unsigned)((K8 / 32 + 1 + 1) / 2)), 64, 0, st>>>(X, R, K, K8, rv, kv, s, mb, sl, ex);
+        if (kv.n == 1) oz::k_split_cols<true><<<blocks, 64, 0, st>>>(X, R, K, K8, rv, kv, s, mb, sl, ex, kspan, kgroups);
+        else oz::k_split_cols<false><<<blocks, 64, 0, st>>>(X, R, K, K8, rv, kv, s, mb, sl, ex, kspan, kgroups);
     }
     return cudaGetLastError();
 }
