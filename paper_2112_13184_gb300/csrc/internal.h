@@ -16,9 +16,8 @@ extern std::atomic<long long> g_launches;
 
 // ---- launch wrappers (kernels.cu) ----------------------------------------
 // All return cudaGetLastError() of their launch; work on `s`.
-// ws (optional): split-K partials when the output has few tiles and K is long;
-// dgemm_splitk_ws_doubles gives the size it wants (0 = no split).
-size_t dgemm_splitk_ws_doubles(int M, int N, int K);
+// ws (optional): split-K partials when the output has few tiles and K is long
+// (splits that do not fit are not taken).
 cudaError_t dgemm(bool tA, bool tB, int M, int N, int K, double alpha, const double* A, int lda,
                   const double* B, int ldb, double beta, double* C, int ldc, cudaStream_t s,
                   double* ws = nullptr, size_t ws_doubles = 0);

@@ -2,6 +2,7 @@
 // normalisation, counter-based Gaussian numbers.  GB300 (sm_103a).
 #include <cuda_runtime.h>
 #include <algorithm>
+#include <cmath>
 #include <cstdint>
 
 #include "internal.h"
@@ -12,79 +13,99 @@ std::atomic<long long> g_launches{0};
 
 // ---------------------------------------------------------------------------
 // FP64 GEMM, row-major: C[M,N] = alpha op(A) op(B) + beta C.
-// 64x64 tile, K-step 16, 256 threads, 4x4 outputs per thread strided by 16
-// so that shared-memory reads broadcast without bank conflicts.  On GB300
-// the FP64 pipe, not memory, bounds this kernel.
+// GB300 issues an FP64 instruction over 64 cycles per SM quarter, so that
+// multiply-adds on padding and idle SMs are all that costs: a few loads per
+// multiply-add do not.  Tiles are therefore small and fitted to the shape:
+// (32 TM) x (8 TN), TM <= 4, TN <= 9, 256 threads of TM x TN outputs each, K
+// taken exactly, next K step prefetched in registers; dgemm_plan picks the
+// tile and a split of K by the work of the fullest SM.  64 x 64 tiles padded
+// N = 36 and 72 to 64 and 128 (the corners of D = 6) and left 144 x 144
+// products on 9 SMs: 144^3 156 -> 15 us, an FP64 sweep at d=2, D=6, chi=48 (all
+// its products) 293 -> 146 ms, at d=2, D=3, chi=16 51 -> 6.5 ms.
 // ---------------------------------------------------------------------------
 namespace {
-constexpr int GB = 64, GK = 16;
+constexpr int GK = 16;
+constexpr int GMAX_TM = 4, GMAX_TN = 9;
 
 // Split-K: blockIdx.z takes K range [z*kchunk, (z+1)*kchunk) and writes its
 // partial product (alpha=1, beta=0) to C + z*zstride; a second kernel sums
 // the partials in fixed order, so results do not depend on scheduling.
-template <bool TA, bool TB>
-__global__ void __launch_bounds__(256) k_dgemm(int M, int N, int K, double alpha,
-                                               const double* __restrict__ A, int lda,
-                                               const double* __restrict__ B, int ldb, double beta,
-                                               double* __restrict__ C, int ldc, int kchunk, size_t zstride) {
+// A element (m, k) at A[m * sam + k * sak], B element (k, n) at B[k * sbk + n * sbn].
+template <int TM, int TN>
+__global__ void __launch_bounds__(256) k_dgemm(int M, int N, int K, double alpha, const double* __restrict__ A,
+                                               long long sam, long long sak, const double* __restrict__ B,
+                                               long long sbk, long long sbn, double beta, double* __restrict__ C,
+                                               int ldc, int kchunk, size_t zstride) {
+    constexpr int BM = 32 * TM, BN = 8 * TN;
+    constexpr int NA = BM * GK / 256, NB = (BN * GK + 255) / 256;
+    __shared__ double As[GK][BM + 1];
+    __shared__ double Bs[GK][BN + 1];
     const int kbeg = blockIdx.z * kchunk;
     const int kend = min(K, kbeg + kchunk);
     C += blockIdx.z * zstride;
-    __shared__ double As[GK][GB + 1];
-    __shared__ double Bs[GK][GB + 1];
-    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-    const long long m0 = (long long)blockIdx.x * GB, n0 = (long long)blockIdx.y * GB;
-    double acc[4][4];
+    const int tid = threadIdx.x, tx = tid & 7, ty = tid >> 3;
+    const long long m0 = (long long)blockIdx.x * BM, n0 = (long long)blockIdx.y * BN;
+    // neighbouring threads load along the contiguous direction
+    const bool a_k = sak == 1, b_k = sbk == 1;
+    double acc[TM][TN];
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+    for (int i = 0; i < TM; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = 0.0;
-
+        for (int j = 0; j < TN; ++j) acc[i][j] = 0.0;
+    double pa[NA], pb[NB];
+    auto load = [&](int k0) {
+#pragma unroll
+        for (int r = 0; r < NA; ++r) {
+            const int idx = tid + 256 * r;
+            const int mm = a_k ? idx / GK : idx % BM, kk = a_k ? idx % GK : idx / BM;
+            pa[r] = (m0 + mm < M && k0 + kk < kend) ? __ldg(A + (m0 + mm) * sam + (long long)(k0 + kk) * sak) : 0.0;
+        }
+#pragma unroll
+        for (int r = 0; r < NB; ++r) {
+            const int idx = tid + 256 * r;
+            const int nn = b_k ? idx / GK : idx % BN, kk = b_k ? idx % GK : idx / BN;
+            pb[r] = (idx < BN * GK && n0 + nn < N && k0 + kk < kend)
+                        ? __ldg(B + (long long)(k0 + kk) * sbk + (n0 + nn) * sbn)
+                        : 0.0;
+        }
+    };
+    if (kbeg < kend) load(kbeg);
     for (int k0 = kbeg; k0 < kend; k0 += GK) {
-#pragma unroll
-        for (int r = 0; r < 4; ++r) {
-            const int idx = tid + 256 * r;
-            int mm, kk;
-            if (!TA) { mm = idx >> 4; kk = idx & 15; } else { mm = idx & 63; kk = idx >> 6; }
-            const long long gm = m0 + mm;
-            const int gk = k0 + kk;
-            double v = 0.0;
-            if (gm < M && gk < kend) v = TA ? A[(size_t)gk * lda + gm] : A[(size_t)gm * lda + gk];
-            As[kk][mm] = v;
-        }
-#pragma unroll
-        for (int r = 0; r < 4; ++r) {
-            const int idx = tid + 256 * r;
-            int nn, kk;
-            if (!TB) { nn = idx & 63; kk = idx >> 6; } else { nn = idx >> 4; kk = idx & 15; }
-            const long long gn = n0 + nn;
-            const int gk = k0 + kk;
-            double v = 0.0;
-            if (gn < N && gk < kend) v = TB ? B[(size_t)gn * ldb + gk] : B[(size_t)gk * ldb + gn];
-            Bs[kk][nn] = v;
-        }
         __syncthreads();
 #pragma unroll
-        for (int kk = 0; kk < GK; ++kk) {
-            double a[4], b[4];
+        for (int r = 0; r < NA; ++r) {
+            const int idx = tid + 256 * r;
+            const int mm = a_k ? idx / GK : idx % BM, kk = a_k ? idx % GK : idx / BM;
+            As[kk][mm] = pa[r];
+        }
 #pragma unroll
-            for (int i = 0; i < 4; ++i) a[i] = As[kk][ty + 16 * i];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) b[j] = Bs[kk][tx + 16 * j];
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
+        for (int r = 0; r < NB; ++r) {
+            const int idx = tid + 256 * r;
+            const int nn = b_k ? idx / GK : idx % BN, kk = b_k ? idx % GK : idx / BN;
+            if (idx < BN * GK) Bs[kk][nn] = pb[r];
         }
         __syncthreads();
+        if (k0 + GK < kend) load(k0 + GK);
+        const int nk = min(GK, kend - k0);
+        for (int kk = 0; kk < nk; ++kk) {
+            double a[TM], b[TN];
+#pragma unroll
+            for (int i = 0; i < TM; ++i) a[i] = As[kk][ty + 32 * i];
+#pragma unroll
+            for (int j = 0; j < TN; ++j) b[j] = Bs[kk][tx + 8 * j];
+#pragma unroll
+            for (int i = 0; i < TM; ++i)
+#pragma unroll
+                for (int j = 0; j < TN; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
+        }
     }
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const long long gm = m0 + ty + 16 * i;
+    for (int i = 0; i < TM; ++i) {
+        const long long gm = m0 + ty + 32 * i;
         if (gm >= M) continue;
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const long long gn = n0 + tx + 16 * j;
+        for (int j = 0; j < TN; ++j) {
+            const long long gn = n0 + tx + 8 * j;
             if (gn >= N) continue;
             double* c = C + (size_t)gm * ldc + gn;
             const double v = alpha * acc[i][j];
@@ -97,6 +118,7 @@ __global__ void k_splitk_reduce(const double* __restrict__ P, int splits, int M,
     const size_t total = (size_t)M * N;
     for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < total; t += (size_t)gridDim.x * blockDim.x) {
         double acc = 0.0;
+#pragma unroll 8
         for (int z = 0; z < splits; ++z) acc += P[(size_t)z * total + t];
         const size_t r = t / N, c = t % N;
         double* cp = C + r * ldc + c;
@@ -104,53 +126,156 @@ __global__ void k_splitk_reduce(const double* __restrict__ P, int splits, int M,
     }
 }
 
-template <bool TA, bool TB>
-void launch(dim3 g, cudaStream_t s, int M, int N, int K, double alpha, const double* A, int lda, const double* B,
-            int ldb, double beta, double* C, int ldc, int kchunk, size_t zs) {
+// A few rows times one vector over a long K (the one-site density matrix: d^2
+// rows of chi^2 D^4): bound by reading A once.  Every CTA takes a K range and
+// all rows; the partials [CTA][row] are summed by one warp per row in fixed
+// order.  At d=3, D=8, chi=128 (9 x 1 x 67M; one 64 x 64 tile split 304 ways
+// before) the one-site density matrix went from 463 to 23 ms.  Shorter K, and
+// calls without a workspace, stay with the tiles.
+constexpr int GEMV_ROWS = 16;
+constexpr int GEMV_CTAS = 152 * 4;
+__global__ void __launch_bounds__(256) k_gemv_long(int M, int K, const double* __restrict__ A, int lda,
+                                                   const double* __restrict__ x, int incx, double* __restrict__ P) {
+    __shared__ double sm[8][GEMV_ROWS];
+    double acc[GEMV_ROWS];
+#pragma unroll
+    for (int m = 0; m < GEMV_ROWS; ++m) acc[m] = 0.0;
+    for (long long k = blockIdx.x * 256ll + threadIdx.x; k < K; k += (long long)gridDim.x * 256) {
+        const double xv = __ldg(x + k * incx);
+#pragma unroll
+        for (int m = 0; m < GEMV_ROWS; ++m)
+            if (m < M) acc[m] = fma(__ldg(A + (size_t)m * lda + k), xv, acc[m]);
+    }
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+#pragma unroll
+    for (int m = 0; m < GEMV_ROWS; ++m) {
+        if (m < M) {
+            for (int o = 16; o > 0; o >>= 1) acc[m] += __shfl_xor_sync(0xffffffffu, acc[m], o);
+            if (lane == 0) sm[w][m] = acc[m];
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x < M) {
+        double t = 0.0;
+        for (int i = 0; i < 8; ++i) t += sm[i][threadIdx.x];
+        P[(size_t)blockIdx.x * M + threadIdx.x] = t;
+    }
+}
+
+__global__ void k_gemv_sum(const double* __restrict__ P, int parts, int M, double alpha, double beta,
+                           double* __restrict__ C, int ldc) {
+    const int m = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    double t = 0.0;
+#pragma unroll 4
+    for (int z = lane; z < parts; z += 32) t += P[(size_t)z * M + m];
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    if (lane == 0) {
+        double* cp = C + (size_t)m * ldc;
+        *cp = (beta == 0.0) ? alpha * t : fma(beta, *cp, alpha * t);
+    }
+}
+
+struct GemmPlan {
+    int tm = 1, tn = 1, splits = 1, kchunk = 1;
+};
+// The tile and K split with the least work on the fullest SM: TM TN multiply-
+// adds per thread and k, at ~150 cycles each (8 warps on 4 quarters, measured
+// 153), an estimated 3000 cycles of launch, fill and drain per CTA, 600 per 16
+// of K for loads that a small tile does not cover, and for a split its
+// partials' pass.
+GemmPlan dgemm_plan(int M, int N, int K, size_t ws_doubles) {
+    GemmPlan best;
+    double best_cost = -1.0;
+    for (int tm = 1; tm <= GMAX_TM; tm *= 2)
+        for (int tn = 1; tn <= GMAX_TN; ++tn) {
+            const double tiles = std::ceil(M / (32.0 * tm)) * std::ceil(N / (8.0 * tn));
+            if (tn < GMAX_TN && N > 8 * tn * 65535) continue;  // grid.y
+            for (int sp = 1; sp <= 256; sp *= 2) {
+                const int kc = ((K + sp - 1) / sp + GK - 1) / GK * GK;
+                const int s = (K + kc - 1) / kc;
+                if (sp > 1 && (s != sp || (size_t)s * M * N > ws_doubles)) break;
+                const double steps = std::ceil(kc / (double)GK), per = (double)tm * tn * std::min(kc, K) * 150.0;
+                const double cta = std::max(per, 600.0 * steps) + 300.0 * steps + 3000.0;
+                const double cost = std::ceil(tiles * s / 152.0) * cta + (s > 1 ? 6000.0 + 40.0 * s * M * N / 152.0 / 32.0 : 0.0);
+                if (best_cost < 0.0 || cost < best_cost) {
+                    best_cost = cost;
+                    best.tm = tm;
+                    best.tn = tn;
+                    best.splits = s;
+                    best.kchunk = kc;
+                }
+            }
+        }
+    return best;
+}
+
+struct GemmArgs64 {
+    int M, N, K;
+    double alpha;
+    const double* A;
+    long long sam, sak;
+    const double* B;
+    long long sbk, sbn;
+    double beta;
+    double* C;
+    int ldc, kchunk;
+    size_t zs;
+};
+template <int TM, int TN>
+void launch(dim3 g, cudaStream_t s, const GemmArgs64& a) {
     ++g_launches;
-    k_dgemm<TA, TB><<<g, 256, 0, s>>>(M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, kchunk, zs);
+    k_dgemm<TM, TN><<<g, 256, 0, s>>>(a.M, a.N, a.K, a.alpha, a.A, a.sam, a.sak, a.B, a.sbk, a.sbn, a.beta, a.C, a.ldc,
+                                      a.kchunk, a.zs);
+}
+template <int TM>
+void launch_tn(int tn, dim3 g, cudaStream_t s, const GemmArgs64& a) {
+    switch (tn) {
+        case 1: launch<TM, 1>(g, s, a); break;
+        case 2: launch<TM, 2>(g, s, a); break;
+        case 3: launch<TM, 3>(g, s, a); break;
+        case 4: launch<TM, 4>(g, s, a); break;
+        case 5: launch<TM, 5>(g, s, a); break;
+        case 6: launch<TM, 6>(g, s, a); break;
+        case 7: launch<TM, 7>(g, s, a); break;
+        case 8: launch<TM, 8>(g, s, a); break;
+        default: launch<TM, 9>(g, s, a); break;
+    }
 }
 }  // namespace
-
-size_t dgemm_splitk_ws_doubles(int M, int N, int K) {
-    const long long tiles = (long long)((M + GB - 1) / GB) * ((N + GB - 1) / GB);
-    if (tiles >= 152 || K < 512) return 0;
-    long long splits = std::min<long long>((304 + tiles - 1) / tiles, K / 256);
-    if (splits < 2) return 0;
-    return (size_t)splits * M * N;
-}
 
 cudaError_t dgemm(bool tA, bool tB, int M, int N, int K, double alpha, const double* A, int lda,
                   const double* B, int ldb, double beta, double* C, int ldc, cudaStream_t s, double* ws,
                   size_t ws_doubles) {
     if (M <= 0 || N <= 0) return cudaSuccess;
-    dim3 grid((unsigned)((M + GB - 1) / GB), (unsigned)((N + GB - 1) / GB), 1);
-    if (grid.y > 65535u) return cudaErrorInvalidValue;
-    const size_t need = dgemm_splitk_ws_doubles(M, N, K);
-    int splits = 1, kchunk = K > 0 ? K : 1;
-    double* out = C;
-    int ldo = ldc;
-    double a = alpha, b = beta;
-    if (need && ws && need <= ws_doubles) {
-        splits = (int)(need / ((size_t)M * N));
-        kchunk = ((K + splits - 1) / splits + GK - 1) / GK * GK;
-        splits = (K + kchunk - 1) / kchunk;
-        grid.z = splits;
-        out = ws;
-        ldo = N;
-        a = 1.0;
-        b = 0.0;
+    if (N == 1 && !tA && M <= GEMV_ROWS && K >= (1 << 16) && ws && ws_doubles >= (size_t)GEMV_CTAS * M) {
+        ++g_launches;
+        k_gemv_long<<<GEMV_CTAS, 256, 0, s>>>(M, K, A, lda, B, tB ? 1 : ldb, ws);
+        ++g_launches;
+        k_gemv_sum<<<1, 32 * M, 0, s>>>(ws, GEMV_CTAS, M, alpha, beta, C, ldc);
+        return cudaGetLastError();
     }
-    const size_t zs = (size_t)M * N;
-    if (!tA && !tB) launch<false, false>(grid, s, M, N, K, a, A, lda, B, ldb, b, out, ldo, kchunk, zs);
-    else if (tA && !tB) launch<true, false>(grid, s, M, N, K, a, A, lda, B, ldb, b, out, ldo, kchunk, zs);
-    else if (!tA && tB) launch<false, true>(grid, s, M, N, K, a, A, lda, B, ldb, b, out, ldo, kchunk, zs);
-    else launch<true, true>(grid, s, M, N, K, a, A, lda, B, ldb, b, out, ldo, kchunk, zs);
-    if (splits > 1) {
-        size_t blocks = (zs + 255) / 256;
+    const GemmPlan p = dgemm_plan(M, N, K, ws ? ws_doubles : 0);
+    const dim3 grid((unsigned)((M + 32 * p.tm - 1) / (32 * p.tm)), (unsigned)((N + 8 * p.tn - 1) / (8 * p.tn)),
+                    (unsigned)p.splits);
+    if (grid.y > 65535u) return cudaErrorInvalidValue;
+    GemmArgs64 a{M, N, K, alpha, A, tA ? 1 : lda, tA ? lda : 1, B, tB ? 1 : ldb, tB ? ldb : 1, beta, C, ldc,
+                 p.splits > 1 ? p.kchunk : std::max(K, 1), (size_t)M * N};
+    if (p.splits > 1) {
+        a.C = ws;
+        a.ldc = N;
+        a.alpha = 1.0;
+        a.beta = 0.0;
+    }
+    switch (p.tm) {
+        case 1: launch_tn<1>(p.tn, grid, s, a); break;
+        case 2: launch_tn<2>(p.tn, grid, s, a); break;
+        default: launch_tn<4>(p.tn, grid, s, a); break;
+    }
+    if (p.splits > 1) {
+        size_t blocks = ((size_t)M * N + 255) / 256;
         if (blocks > 152 * 8) blocks = 152 * 8;
         ++g_launches;
-        k_splitk_reduce<<<(unsigned)blocks, 256, 0, s>>>(ws, splits, M, N, alpha, beta, C, ldc);
+        k_splitk_reduce<<<(unsigned)blocks, 256, 0, s>>>(ws, p.splits, M, N, alpha, beta, C, ldc);
     }
     return cudaGetLastError();
 }
