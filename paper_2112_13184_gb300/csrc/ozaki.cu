@@ -28,6 +28,7 @@
 #include <cudaTypedefs.h>
 
 #include <algorithm>
+#include <cmath>
 #include <cstdint>
 #include <mutex>
 
@@ -153,30 +154,52 @@ __device__ __forceinline__ double i64_ldexp(long long Z, int E) {
     return __longlong_as_double((long long)((neg << 63) | ((unsigned long long)be << 52) | (mant & ((1ull << 52) - 1))));
 }
 
-// round(f * 2^k) as int64 from the FP32 bit pattern (|f 2^k| < 2^62)
-__device__ __forceinline__ long long f32_fixed(float f, int k) {
-    const unsigned b = __float_as_uint(f);
-    const int ex = (int)((b >> 23) & 0xff);
-    if (ex == 0) return 0;  // zero or FP32 denormal: far below the resolution kept
-    const long long mant = (long long)((b & 0x7fffff) | 0x800000);
-    const int sh = ex - 150 + k;  // f 2^k = mant 2^sh
-    long long v;
-    if (sh >= 0) v = mant << sh;
-    else if (sh <= -25) v = 0;
-    else v = (mant + (1ll << (-sh - 1))) >> (-sh);
-    return (b >> 31) ? -v : v;
+// C = 2^(eA+eB-16) (S0 + S1/256 + F): with F kept to 2^-28 of an S0 unit (below
+// 2^-44 of max|row| max|col|), Z = 2^28 S0 + 2^20 S1 + round(2^28 F) is an
+// exact int64 (one K chunk: |Z| < 2^53; 64 chunks: < 2^59) and C = Z
+// 2^(eA+eB-44).  S0 and S1/256 are whole-numbered FP32 accumulators; F, below
+// 2^9 per chunk, is split by two magic additions of 1.5 2^23 into 6 and 22
+// fractional bits: no conversion of it (an FP32 -> int64 conversion issues on
+// the FP64 pipe, 64 cycles a warp; FP32 -> int32 on the 16-lane one).
+__device__ __forceinline__ long long fixed_add(long long Z, float a0, float a1, float F) {
+    const float h = fmaf(F, 64.0f, 12582912.0f);
+    const float r = fmaf(F, 64.0f, 12582912.0f - h);  // F 2^6 minus its rounding, exact
+    const float h2 = fmaf(r, 4194304.0f, 12582912.0f);
+    const int i1 = __float_as_int(h) - 0x4B400000, i2 = __float_as_int(h2) - 0x4B400000;
+    Z += i2;
+    Z += (long long)i1 * (1 << 22);
+    Z += (long long)__float2int_rn(a1 * 256.0f) * (1 << 20);
+    Z += (long long)__float2int_rn(a0) * (1 << 28);
+    return Z;
 }
-
-// C = 2^(eA+eB-16) (S0 + S1/256 + F).  With T = 256 S0 + S1 (exact; |T| <
-// 2^39 for K <= 16384 per split) and F kept to 2^-28 of an S0 unit (below
-// 2^-44 of max|row| max|col|), Z = 2^20 T + round(2^28 F) is an exact int64
-// and C = Z 2^(eA+eB-44).  escale = eA + eB - 16.  round(2^28 F) is taken
-// from F's bit pattern: an FP32 -> int64 conversion instruction issues on
-// the FP64 pipe, which GB300 runs at 2 lanes per clock per SM.
-__device__ __forceinline__ double assemble(int S0, int S1, float F, int escale) {
-    const long long T = (long long)S0 * 256 + (long long)S1;
-    const long long Z = T * (1ll << 20) + f32_fixed(F, 28);  // F 2^28 < 2^62
-    return i64_ldexp(Z, escale - 28);
+// exponents of rows with an infinity or a NaN (1025) become one that leaves
+// the FP64 range from any finite partner
+constexpr int BAD_EXP = 100000;
+__device__ __forceinline__ int safe_exp(int e) { return e > 1024 ? BAD_EXP : e; }
+// Z 2^E where |Z| < 2^53 (exact: a left shift only) and the result is normal
+// or zero; else `bad` is set and the value is meaningless.  No branch: a
+// branch per entry kept the entries of a block from overlapping.
+__device__ __forceinline__ double z_scaled_fast(long long Z, int E, bool& bad) {
+    const long long sg = Z >> 63;
+    const unsigned long long m = (unsigned long long)((Z ^ sg) - sg);
+    const unsigned mh = (unsigned)(m >> 32), ml = (unsigned)m;
+    const int c = mh ? __clz((int)mh) : 32 + __clz((int)ml);
+    const int be = c == 64 ? 1 : E + 1086 - c;  // biased exponent of m 2^E; 1 makes a zero come out as zero
+    bad = bad || c < 11 || (unsigned)(be - 1) >= 2046u || E > BAD_EXP / 2;
+    const unsigned long long mant = m << ((c - 11) & 63);  // implicit bit at 52
+    const unsigned hi = (unsigned)(mant >> 32) + ((unsigned)(be - 1) << 20) + ((unsigned)sg & 0x80000000u);
+    return __hiloint2double((int)hi, (int)(unsigned)mant);
+}
+// larger |Z| (sums of several chunks), results outside the normal range,
+// non-finite operands
+__device__ __noinline__ double z_scaled_slow(long long Z, int E) {
+    if (E > BAD_EXP / 2) return __longlong_as_double(0x7ff8000000000000ll);
+    return i64_ldexp(Z, E);
+}
+__device__ __forceinline__ double z_scaled(long long Z, int E) {
+    bool bad = false;
+    const double v = z_scaled_fast(Z, E, bad);
+    return bad ? z_scaled_slow(Z, E) : v;
 }
 
 __device__ __noinline__ double f32_ldexp_slow(float f, int E) { return ldexp((double)f, E); }
@@ -733,6 +756,17 @@ __device__ __forceinline__ void tc_ld16(uint32_t taddr, uint32_t* r) {
           "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
         : "r"(taddr));
 }
+__device__ __forceinline__ void tc_ld8(uint32_t taddr, uint32_t* r) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+        : "r"(taddr));
+}
+// four doubles to a 32-byte aligned address: a whole sector per lane
+__device__ __forceinline__ void st_global4(double* p, const double* v) {
+    asm volatile("st.global.v4.f64 [%0], {%1, %2, %3, %4};" ::"l"(p), "d"(v[0]), "d"(v[1]), "d"(v[2]), "d"(v[3])
+                 : "memory");
+}
 __device__ __forceinline__ void tc_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
 // Shared-memory matrix descriptor of a K-major, 64-byte-swizzled tile
@@ -748,13 +782,55 @@ __device__ __forceinline__ uint64_t sw64_desc(uint32_t saddr) {
 }
 
 
+// one thread of a converged warp (the same one at every call)
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
+    return p != 0;
+}
+// tc_mma on descriptors given by their low words (address, leading offset)
+__device__ __forceinline__ void tc_mma_lo(uint32_t d_tmem, uint32_t alo, uint32_t blo, uint32_t hi, uint32_t idesc,
+                                          uint32_t accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\t"
+        "mov.b64 da, {%1, %3};\n\tmov.b64 db, {%2, %3};\n\t"
+        "setp.ne.b32 p, %5, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, p;\n\t}" ::"r"(d_tmem),
+        "r"(alo), "r"(blo), "r"(hi), "r"(idesc), "r"(accumulate)
+        : "memory");
+}
+// All slice products of one 32-wide k-block, S slices: level 0 and level 1 into
+// their accumulators, the rest into the third; keep = 0 restarts the three.
+// Straight-line code on constant offsets from the two tile addresses: issued
+// from loops over runtime slice indices an MMA took 137 cycles whatever its
+// width, so ~100 at N = 144 and 75 at N = 64.
+template <int S, int BN>
+__device__ __forceinline__ void issue_levels(uint32_t tmem, uint32_t sa, uint32_t sb, uint32_t idesc, uint32_t keep) {
+    constexpr uint64_t top = (uint64_t)(512 >> 4) << 32 | (uint64_t)1 << 46 | (uint64_t)4 << 61;  // as sw64_desc
+    constexpr uint32_t hi = (uint32_t)(top >> 32);
+    const uint32_t a0 = (sa >> 4) | (1u << 16), b0 = (sb >> 4) | (1u << 16);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {  // two K=16 halves, 32 bytes apart in the 64-byte row
+        const uint32_t k0 = h ? 1u : keep;
+        tc_mma_lo(tmem, a0 + 2 * h, b0 + 2 * h, hi, idesc, k0);
+        tc_mma_lo(tmem + BN, a0 + 2 * h, b0 + BN * 4 + 2 * h, hi, idesc, k0);
+        tc_mma_lo(tmem + BN, a0 + BM * 4 + 2 * h, b0 + 2 * h, hi, idesc, 1u);
+#pragma unroll
+        for (int L = 2; L < S; ++L)
+#pragma unroll
+            for (int t = 0; t <= L; ++t)
+                tc_mma_lo(tmem + 2 * BN, a0 + t * (BM * 4) + 2 * h, b0 + (L - t) * (BN * 4) + 2 * h, hi, idesc,
+                          (L == 2 && t == 0) ? k0 : 1u);
+    }
+}
+
 // ---------------------------------------------------------------------------
 // slice GEMM
 // ---------------------------------------------------------------------------
 struct GemmArgs {
     int M, N;             // logical output size
     int nkb;              // 32-wide k-blocks in K
-    int kb_per_split;     // k-blocks per blockIdx.z (a multiple of CHUNK_KB)
+    int kb_per_split;     // k-blocks per blockIdx.z
     int s;                // slices per operand
     int stages;
     uint32_t a_bytes, stage_bytes;
@@ -764,24 +840,78 @@ struct GemmArgs {
     double alpha, beta;
     double* C;
     View out_r, out_c;    // C offset of (m, n) = view(out_r, m) + view(out_c, n)
-    int* PS0;             // split-K partials [z][Mpad][Npad]
-    int* PS1;
-    float* PF;
+    int plain;            // alpha = 1 and beta = 0
+    int vec;              // 4 or 2: aligned groups of so many columns are contiguous; else 1
+    long long* PZ;        // split-K partials [z][Mpad][Npad]
     int Mpad, Npad;
     int m_tiles, n_tiles;
     int* err;
     long long wait_limit; // cycles before a bounded wait gives up
 };
 
-// ONE: every CTA's K range is a single chunk (every corner product), so no
-// sum is carried across chunks; a separate instantiation keeps the
-// multi-chunk sums' registers out of that path.
+// Eight consecutive output columns from n8 of the lane's row m: built from
+// their int64 sums and stored (crow: the row's output address, ea = row
+// exponent - 44; every lane of the warp calls).
+__device__ __forceinline__ void emit8(const GemmArgs& g, const long long* Z, int ea, int m, int n8, double* crow,
+                                      int lane) {
+    // the columns are the same for every lane: lane j works out column j's
+    // offset and exponent once
+    const int nl = n8 + (lane & 7);
+    const unsigned coff_l = nl < g.N ? (unsigned)view_offset32(g.out_c, (unsigned)nl) : 0u;
+    const int eb_l = nl < g.N ? safe_exp(g.eB[nl]) : 0;
+    double v[8];
+    bool bad = false;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) v[j] = z_scaled_fast(Z[j], ea + __shfl_sync(0xffffffffu, eb_l, j), bad);
+    if (__any_sync(0xffffffffu, bad)) {
+#pragma unroll
+        for (int j = 0; j < 8; ++j) v[j] = z_scaled(Z[j], ea + __shfl_sync(0xffffffffu, eb_l, j));
+    }
+    const bool row = m < g.M;
+    // alpha = 1, beta = 0 (every product of the sweep): no FP64 arithmetic at
+    // all; the branches are uniform, so nothing is issued under a predicate
+    if (g.plain && n8 + 8 <= g.N) {
+        if (g.vec == 4) {
+            const unsigned c0 = __shfl_sync(0xffffffffu, coff_l, 0), c4 = __shfl_sync(0xffffffffu, coff_l, 4);
+            if (row) {
+                st_global4(crow + c0, v);
+                st_global4(crow + c4, v + 4);
+            }
+        } else if (g.vec == 2) {
+#pragma unroll
+            for (int j = 0; j < 8; j += 2) {
+                const unsigned c = __shfl_sync(0xffffffffu, coff_l, j);
+                if (row) *reinterpret_cast<double2*>(crow + c) = make_double2(v[j], v[j + 1]);
+            }
+        } else {
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                const unsigned c = __shfl_sync(0xffffffffu, coff_l, j);
+                if (row) crow[c] = v[j];
+            }
+        }
+        return;
+    }
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+        const unsigned c = __shfl_sync(0xffffffffu, coff_l, j);
+        if (!row || n8 + j >= g.N) continue;
+        double* cp = crow + c;
+        if (g.plain) {
+            *cp = v[j];
+        } else {
+            const double w = v[j] * g.alpha;
+            *cp = g.beta == 0.0 ? w : fma(g.beta, *cp, w);
+        }
+    }
+}
+
 // MODE 0: exact-level emulated FP64 (above).  MODE 1: split-BF16 -- the same
 // BF16 digit slices, every product of levels <= s-1 accumulated in one FP32
 // accumulator over all of K.  MODE 2: 3xTF32 -- two TF32 slices (base-2^11
 // digits), hi*hi + hi*lo + lo*hi on kind::tf32 into one FP32 accumulator.
 // Modes 1 and 2 run without split-K and read TMEM once per tile.
-template <int NB16, bool ONE, int MODE>
+template <int NB16, int MODE>
 __global__ void __launch_bounds__(THREADS, 1)
     k_oz_gemm(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const GemmArgs g) {
     constexpr int BN = 16 * NB16;
@@ -870,7 +1000,9 @@ __global__ void __launch_bounds__(THREADS, 1)
         }
     } else if (warp == EPI_WARPS + 1) {
         // ---------------- MMA issuer ----------------
-        if (lane == 0) {
+        // the warp stays converged and elects the issuing thread per k-block:
+        // addresses then live in uniform registers
+        {
             // D format F32 (1); A and B both BF16 (1) under kind::f16, both TF32 (2) under kind::tf32
             constexpr uint32_t fmt = MODE == 2 ? 2u : 1u;
             const uint32_t idesc = (1u << 4) | (fmt << 7) | (fmt << 10) | ((uint32_t)(BN >> 3) << 17) |
@@ -883,56 +1015,54 @@ __global__ void __launch_bounds__(THREADS, 1)
                 const uint32_t ph = (uint32_t)(it / g.stages) & 1u;
                 const bool first = MODE == 0 ? (i % CHUNK_KB) == 0 : i == 0;
                 const bool last = MODE == 0 ? ((i % CHUNK_KB) == CHUNK_KB - 1 || i == nkb - 1) : i == nkb - 1;
-                if (first && cc > 0 && !mbar_wait(acc_empty, (uint32_t)(cc - 1) & 1u, g.err, g.wait_limit)) {
-                    ok = false;
-                    break;
-                }
-                if (!mbar_wait(&full[st], ph, g.err, g.wait_limit)) {
+                bool go = !(first && cc > 0) || mbar_wait(acc_empty, (uint32_t)(cc - 1) & 1u, g.err, g.wait_limit);
+                go = go && mbar_wait(&full[st], ph, g.err, g.wait_limit);
+                if (!__all_sync(0xffffffffu, go)) {
                     ok = false;
                     break;
                 }
                 tc_fence_after();
                 const uint32_t sa = base + (uint32_t)st * g.stage_bytes;
                 const uint32_t sb = sa + g.a_bytes;
-                if (MODE != 0) {
-                    // two 32-byte K halves (16 BF16 or 8 TF32 each); every level
-                    // <= s-1 into the one FP32 accumulator
-                    for (int h = 0; h < 2; ++h) {
-                        bool f1 = first && h == 0;
-                        for (int L = 0; L < g.s; ++L)
-                            for (int t = 0; t <= L; ++t) {
-                                const uint64_t ad = sw64_desc(sa + t * (BM * 64) + h * 32);
-                                const uint64_t bd = sw64_desc(sb + (L - t) * (BN * 64) + h * 32);
-                                if (MODE == 2) tc_mma_tf32(tmem, ad, bd, idesc, f1 ? 0u : 1u);
-                                else tc_mma(tmem, ad, bd, idesc, f1 ? 0u : 1u);
-                                f1 = false;
-                            }
-                    }
-                } else
-                for (int h = 0; h < 2; ++h) {  // two K=16 halves, 32 bytes apart in the 64-byte row
-                    const uint32_t restart = (first && h == 0) ? 0u : 1u;
-                    tc_mma(tmem, sw64_desc(sa + h * 32), sw64_desc(sb + h * 32), idesc, restart);
-                    tc_mma(tmem + BN, sw64_desc(sa + h * 32), sw64_desc(sb + BN * 64 + h * 32), idesc, restart);
-                    tc_mma(tmem + BN, sw64_desc(sa + BM * 64 + h * 32), sw64_desc(sb + h * 32), idesc, 1u);
-                    bool first2 = first && h == 0;  // the FP32 levels restart every chunk
-                    for (int L = 2; L < g.s; ++L)
-                        for (int t = 0; t <= L; ++t) {
-                            tc_mma(tmem + 2 * BN, sw64_desc(sa + t * (BM * 64) + h * 32),
-                                   sw64_desc(sb + (L - t) * (BN * 64) + h * 32), idesc, first2 ? 0u : 1u);
-                            first2 = false;
+                if (elect_one()) {
+                    if (MODE != 0) {
+                        // two 32-byte K halves (16 BF16 or 8 TF32 each); every level
+                        // <= s-1 into the one FP32 accumulator
+                        for (int h = 0; h < 2; ++h) {
+                            bool f1 = first && h == 0;
+                            for (int L = 0; L < g.s; ++L)
+                                for (int t2 = 0; t2 <= L; ++t2) {
+                                    const uint64_t ad = sw64_desc(sa + t2 * (BM * 64) + h * 32);
+                                    const uint64_t bd = sw64_desc(sb + (L - t2) * (BN * 64) + h * 32);
+                                    if (MODE == 2) tc_mma_tf32(tmem, ad, bd, idesc, f1 ? 0u : 1u);
+                                    else tc_mma(tmem, ad, bd, idesc, f1 ? 0u : 1u);
+                                    f1 = false;
+                                }
                         }
+                    } else {
+                        const uint32_t keep = first ? 0u : 1u;  // the FP32 levels restart every chunk too
+                        switch (g.s) {
+                            case 2: issue_levels<2, BN>(tmem, sa, sb, idesc, keep); break;
+                            case 3: issue_levels<3, BN>(tmem, sa, sb, idesc, keep); break;
+                            case 4: issue_levels<4, BN>(tmem, sa, sb, idesc, keep); break;
+                            case 5: issue_levels<5, BN>(tmem, sa, sb, idesc, keep); break;
+                            default: issue_levels<6, BN>(tmem, sa, sb, idesc, keep); break;
+                        }
+                    }
+                    tc_commit(&empty[st]);
+                    if (last) tc_commit(acc_full);
                 }
-                tc_commit(&empty[st]);
-                if (last) {
-                    tc_commit(acc_full);
-                    ++cc;
+                __syncwarp();
+                if (last) ++cc;
+            }
+            // every MMA issued by this warp completes before TMEM is freed
+            if (elect_one()) {
+                tc_commit(drain);
+                const long long t0 = clock64();
+                while (!mbar_try_wait(drain, 0u) && clock64() - t0 < g.wait_limit) {
                 }
             }
-            // every MMA issued by this thread completes before TMEM is freed
-            tc_commit(drain);
-            const long long t0 = clock64();
-            while (!mbar_try_wait(drain, 0u) && clock64() - t0 < g.wait_limit) {
-            }
+            __syncwarp();
         }
     } else if (MODE != 0) {
         // ---------------- epilogue of the FP32-accumulated modes ----------------
@@ -986,114 +1116,70 @@ __global__ void __launch_bounds__(THREADS, 1)
         }
     } else {
         // ---------------- epilogue: warps 0..11 ----------------
+        // Three warps per TMEM lane quarter share the tile's 8-column blocks.
+        // Every chunk's three accumulators are added to one int64 per entry;
+        // the last chunk's TMEM is released as soon as it is read, so that the
+        // next tile's MMAs run while this tile's results are built and stored.
+        // (Held as two int32 and one FP32 sum, 144 columns took more registers
+        // than there are: the spills cost a K = 8192 product ~16000 cycles per
+        // chunk beside 25000 of MMAs.)
         const int q = warp & 3, grp = warp >> 2;
         const uint32_t lane_addr = tmem + ((uint32_t)(q * 32) << 16);
+        constexpr int NB8 = 2 * NB16, NC = (NB8 + 2) / 3;  // 8-column blocks, most per warp
         int cc = 0;  // accumulator chunks drained so far, over all tiles
         bool ok = true;
-        const bool unit_alpha = g.alpha == 1.0, zero_beta = g.beta == 0.0;
         for (int t = t_first; t < ntiles && ok; t += t_step) {
-        const int m0 = tile_m0(t), n0 = tile_n0(t);
-        const int m = m0 + q * 32 + lane;
-        const int ea = (g.direct && m < g.M) ? g.eA[m] : 0;
-        // Multi-chunk tiles carry the exact level-0/1 sums (int32) and the
-        // sum of the per-chunk FP32 levels across K chunks, and finish each
-        // 16-column block in the last chunk before reading the next.  A
-        // single-chunk tile (every corner product: K <= 256) reads all of
-        // TMEM first and releases it, so that the next tile's MMAs run while
-        // this tile's results are assembled and stored.
-        constexpr int NC = NBG;
-        int S0[NC][16], S1[NC][16];
-        float Fs[NC][16];
+            const int m0 = tile_m0(t), n0 = tile_n0(t);
+            const int m = m0 + q * 32 + lane;
+            const int ea = (g.direct && m < g.M) ? safe_exp(g.eA[m]) - 44 : 0;
+            long long Z[NC][8];
 #pragma unroll
-        for (int jb = 0; jb < NC; ++jb)
+            for (int jb = 0; jb < NC; ++jb)
 #pragma unroll
-            for (int j = 0; j < 16; ++j) S0[jb][j] = S1[jb][j] = 0, Fs[jb][j] = 0.f;
-        // result of column block jb: assembled and stored (direct) or kept
-        // as split-K partials
-        auto finish = [&](int jb) {
-            const int b = grp + 3 * jb;
-            if (g.direct) {
-                // the 16 columns of this block are the same for every lane:
-                // lane j works out column j's offset and exponent once
-                const int nl = n0 + b * 16 + (lane & 15);
-                const long long coff_l = nl < g.N ? view_offset32(g.out_c, (unsigned)nl) : 0;
-                const int eb_l = nl < g.N ? g.eB[nl] : 0;
-                double* crow = g.C + (m < g.M ? view_offset32(g.out_r, (unsigned)m) : 0);
-                // alpha = 1, beta = 0 (every product of the sweep) takes a loop
-                // with no FP64 arithmetic at all: the branch is uniform, so
-                // the scaling is not issued under a predicate per element
-                if (unit_alpha && zero_beta) {
-#pragma unroll
-                    for (int j = 0; j < 16; ++j) {
-                        const long long coff = __shfl_sync(0xffffffffu, coff_l, j);
-                        const int eb = __shfl_sync(0xffffffffu, eb_l, j);
-                        const int n = n0 + b * 16 + j;
-                        if (m >= g.M || n >= g.N) continue;
-                        double v = assemble(S0[jb][j], S1[jb][j], Fs[jb][j], ea + eb - 16);
-                        if (ea > 1024 || eb > 1024) v = __longlong_as_double(0x7ff8000000000000ll);  // non-finite operand
-                        crow[coff] = v;
-                    }
-                } else {
-#pragma unroll
-                    for (int j = 0; j < 16; ++j) {
-                        const long long coff = __shfl_sync(0xffffffffu, coff_l, j);
-                        const int eb = __shfl_sync(0xffffffffu, eb_l, j);
-                        const int n = n0 + b * 16 + j;
-                        if (m >= g.M || n >= g.N) continue;
-                        double v = assemble(S0[jb][j], S1[jb][j], Fs[jb][j], ea + eb - 16);
-                        if (ea > 1024 || eb > 1024) v = __longlong_as_double(0x7ff8000000000000ll);
-                        v *= g.alpha;
-                        double* cp = crow + coff;
-                        *cp = zero_beta ? v : fma(g.beta, *cp, v);
-                    }
+                for (int j = 0; j < 8; ++j) Z[jb][j] = 0;
+            for (int c = 0; c < nchunks; ++c, ++cc) {
+                if (!mbar_wait(acc_full, (uint32_t)cc & 1u, g.err, g.wait_limit)) {
+                    ok = false;
+                    break;
                 }
-            } else {
-                const size_t row = ((size_t)blockIdx.z * g.Mpad + m) * g.Npad + n0 + b * 16;
+                tc_fence_after();
 #pragma unroll
-                for (int j = 0; j < 16; ++j) {
-                    g.PS0[row + j] = S0[jb][j];
-                    g.PS1[row + j] = S1[jb][j];
-                    g.PF[row + j] = Fs[jb][j];
-                }
-            }
-        };
-        for (int c = 0; c < nchunks; ++c, ++cc) {
-            if (!mbar_wait(acc_full, (uint32_t)cc & 1u, g.err, g.wait_limit)) {
-                ok = false;
-                break;
-            }
-            tc_fence_after();
-            const bool last = c == nchunks - 1;
-#pragma unroll
-            for (int jb = 0; jb < NBG; ++jb) {
-                const int b = grp + 3 * jb;
-                if (b >= NB16) continue;
-                uint32_t r0[16], r1[16];
-                tc_ld16(lane_addr + b * 16, r0);
-                tc_ld16(lane_addr + BN + b * 16, r1);
-                tc_wait_ld();
-#pragma unroll
-                for (int j = 0; j < 16; ++j) {
-                    S0[jb][j] += __float2int_rn(__uint_as_float(r0[j]));
-                    S1[jb][j] += __float2int_rn(__uint_as_float(r1[j]) * 256.0f);
-                }
-                if (g.s > 2) {
-                    tc_ld16(lane_addr + 2 * BN + b * 16, r0);
+                for (int jb = 0; jb < NC; ++jb) {
+                    const int b = grp + 3 * jb;
+                    if (b >= NB8) continue;
+                    uint32_t r0[8], r1[8], r2[8];
+                    tc_ld8(lane_addr + b * 8, r0);
+                    tc_ld8(lane_addr + BN + b * 8, r1);
+                    if (g.s > 2) tc_ld8(lane_addr + 2 * BN + b * 8, r2);
                     tc_wait_ld();
 #pragma unroll
-                    for (int j = 0; j < 16; ++j) Fs[jb][j] += __uint_as_float(r0[j]);
+                    for (int j = 0; j < 8; ++j)
+                        Z[jb][j] = fixed_add(Z[jb][j], __uint_as_float(r0[j]), __uint_as_float(r1[j]),
+                                             g.s > 2 ? __uint_as_float(r2[j]) : 0.0f);
                 }
-                if (!ONE && last) finish(jb);
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(acc_empty);
             }
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(acc_empty);
-        }
-        if (ONE && ok) {
+            if (!ok) break;
+            if (g.direct) {
+                double* crow = g.C + (m < g.M ? view_offset32(g.out_r, (unsigned)m) : 0);
 #pragma unroll
-            for (int jb = 0; jb < NBG; ++jb)
-                if (grp + 3 * jb < NB16) finish(jb);
-        }
+                for (int jb = 0; jb < NC; ++jb) {
+                    const int b = grp + 3 * jb;
+                    if (b < NB8) emit8(g, Z[jb], ea, m, n0 + b * 8, crow, lane);
+                }
+            } else {
+#pragma unroll
+                for (int jb = 0; jb < NC; ++jb) {
+                    const int b = grp + 3 * jb;
+                    if (b >= NB8) continue;
+                    longlong2* row = reinterpret_cast<longlong2*>(
+                        g.PZ + ((size_t)blockIdx.z * g.Mpad + m) * g.Npad + n0 + b * 8);
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) row[j] = make_longlong2(Z[jb][2 * j], Z[jb][2 * j + 1]);
+                }
+            }
         }  // tiles
     }
     tc_fence_before();
@@ -1104,24 +1190,196 @@ __global__ void __launch_bounds__(THREADS, 1)
     }
 }
 
-// split-K partials -> C
-__global__ void k_oz_combine(const int* __restrict__ PS0, const int* __restrict__ PS1, const float* __restrict__ PF,
-                             int splits, int Mpad, int Npad, int M, int N, const int* __restrict__ eA,
-                             const int* __restrict__ eB, double alpha, double beta, double* __restrict__ C,
-                             View out_r, View out_c) {
-    const size_t total = (size_t)M * N;
+// Products of a single exact chunk (K <= 256: every product of an enlarged
+// corner), emulated FP64 only.  Their epilogue -- ~70 instructions per entry,
+// half of them on the 16-lane integer pipe -- outweighs the 30 MMAs per
+// 32 of K, and with three warps per SM quarter and one set of accumulators
+// it was bound by latency (38% of issue slots) and waited for the MMAs in
+// between.  Here two teams of twelve warps take turns on two sets of
+// accumulators (BN <= 80: 6 BN <= 480 of 512 TMEM columns): the MMAs of one
+// tile run under the epilogues of the two before it, and a warp holds eight
+// columns at a time, so that 26 warps fit the register file.
+// 262144 x 192 x 64 in its sweep layout: 340 -> 176 us; 8192 x 8192 x 128: 527 -> 278.
+constexpr int TEAM_WARPS = 12;
+constexpr int SHORT_THREADS = (2 * TEAM_WARPS + 2) * 32;
+template <int NB16>
+__global__ void __launch_bounds__(SHORT_THREADS, 1)
+    k_oz_gemm_short(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const GemmArgs g) {
+    constexpr int BN = 16 * NB16;
+    constexpr uint32_t TMEM_COLS = 6 * BN <= 128 ? 128 : 6 * BN <= 256 ? 256 : 512;
+    extern __shared__ uint8_t smem_raw[];
+    const uint32_t raw = smem_u32(smem_raw);
+    const uint32_t base = (raw + 1023u) & ~1023u;
+    uint8_t* sbase = smem_raw + (base - raw);
+    uint64_t* full = (uint64_t*)(sbase + (size_t)g.stages * g.stage_bytes);
+    uint64_t* empty = full + g.stages;
+    uint64_t* acc_full = empty + g.stages;   // [2]
+    uint64_t* acc_empty = acc_full + 2;      // [2]
+    uint64_t* drain = acc_empty + 2;
+    uint32_t* tmem_slot = (uint32_t*)(drain + 1);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int ntiles = g.m_tiles * g.n_tiles, nkb = g.nkb;
+
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
+                     "r"(TMEM_COLS)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    if (threadIdx.x == 32) {
+        for (int st = 0; st < g.stages; ++st) {
+            mbar_init(&full[st], 1);
+            mbar_init(&empty[st], 1);
+        }
+        for (int u = 0; u < 2; ++u) {
+            mbar_init(&acc_full[u], 1);
+            mbar_init(&acc_empty[u], TEAM_WARPS);
+        }
+        mbar_init(drain, 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = *tmem_slot;
+
+    if (warp == 2 * TEAM_WARPS) {
+        // ---------------- TMA producer ----------------
+        if (lane == 0) {
+            int issued = 0;
+            bool ok = true;
+            for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
+                const int m0 = t / g.n_tiles * BM, n0 = t % g.n_tiles * BN;
+                for (int i = 0; i < nkb; ++i) {
+                    const int st = issued % g.stages;
+                    if (!mbar_wait(&empty[st], ((uint32_t)(issued / g.stages) & 1u) ^ 1u, g.err, g.wait_limit)) {
+                        ok = false;
+                        break;
+                    }
+                    uint8_t* sa = sbase + (size_t)st * g.stage_bytes;
+                    mbar_expect_tx(&full[st], g.stage_bytes);
+                    tma_load_3d(sa, &tmA, i * BK, m0, 0, &full[st]);
+                    tma_load_3d(sa + g.a_bytes, &tmB, i * BK, n0, 0, &full[st]);
+                    ++issued;
+                }
+            }
+            if (*(volatile int*)g.err) {
+                // let the copies still in flight land before the CTA exits
+                for (int i = max(0, issued - g.stages); i < issued; ++i) {
+                    const long long t0 = clock64();
+                    while (!mbar_try_wait(&full[i % g.stages], (uint32_t)(i / g.stages) & 1u) &&
+                           clock64() - t0 < g.wait_limit) {
+                    }
+                }
+            }
+        }
+    } else if (warp == 2 * TEAM_WARPS + 1) {
+        // ---------------- MMA issuer (converged warp, one elected thread) ----------------
+        const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
+        int it = 0, ti = 0;
+        bool ok = true;
+        for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x, ++ti) {
+            const int buf = ti & 1;
+            bool go = ti < 2 || mbar_wait(&acc_empty[buf], (uint32_t)((ti >> 1) - 1) & 1u, g.err, g.wait_limit);
+            for (int i = 0; i < nkb; ++i, ++it) {
+                const int st = it % g.stages;
+                go = go && mbar_wait(&full[st], (uint32_t)(it / g.stages) & 1u, g.err, g.wait_limit);
+                if (!__all_sync(0xffffffffu, go)) {
+                    ok = false;
+                    break;
+                }
+                tc_fence_after();
+                const uint32_t sa = base + (uint32_t)st * g.stage_bytes, sb = sa + g.a_bytes;
+                const uint32_t acc = tmem + (uint32_t)buf * (3 * BN), keep = i == 0 ? 0u : 1u;
+                if (elect_one()) {
+                    switch (g.s) {
+                        case 2: issue_levels<2, BN>(acc, sa, sb, idesc, keep); break;
+                        case 3: issue_levels<3, BN>(acc, sa, sb, idesc, keep); break;
+                        case 4: issue_levels<4, BN>(acc, sa, sb, idesc, keep); break;
+                        case 5: issue_levels<5, BN>(acc, sa, sb, idesc, keep); break;
+                        default: issue_levels<6, BN>(acc, sa, sb, idesc, keep); break;
+                    }
+                    tc_commit(&empty[st]);
+                    if (i == nkb - 1) tc_commit(&acc_full[buf]);
+                }
+                __syncwarp();
+            }
+        }
+        // every MMA issued by this warp completes before TMEM is freed
+        if (elect_one()) {
+            tc_commit(drain);
+            const long long t0 = clock64();
+            while (!mbar_try_wait(drain, 0u) && clock64() - t0 < g.wait_limit) {
+            }
+        }
+        __syncwarp();
+    } else {
+        // ---------------- epilogue: two teams of 3 warps per TMEM lane quarter ----------------
+        const int team = warp >= TEAM_WARPS ? 1 : 0, q = warp & 3, grp = (warp - team * TEAM_WARPS) >> 2;
+        constexpr int NB8 = 2 * NB16;
+        const uint32_t lane_addr = tmem + (uint32_t)team * (3 * BN) + ((uint32_t)(q * 32) << 16);
+        int ti = team;
+        for (int t = blockIdx.x + team * gridDim.x; t < ntiles; t += 2 * gridDim.x, ti += 2) {
+            const int m0 = t / g.n_tiles * BM, n0 = t % g.n_tiles * BN;
+            const int m = m0 + q * 32 + lane;
+            const int ea = m < g.M ? safe_exp(g.eA[m]) - 44 : 0;
+            double* crow = g.C + (m < g.M ? view_offset32(g.out_r, (unsigned)m) : 0);
+            if (!mbar_wait(&acc_full[team], (uint32_t)(ti >> 1) & 1u, g.err, g.wait_limit)) break;
+            tc_fence_after();
+            for (int b = grp; b < NB8; b += 3) {
+                uint32_t r0[8], r1[8], r2[8];
+                tc_ld8(lane_addr + b * 8, r0);
+                tc_ld8(lane_addr + BN + b * 8, r1);
+                if (g.s > 2) tc_ld8(lane_addr + 2 * BN + b * 8, r2);
+                tc_wait_ld();
+                if (b + 3 >= NB8) {  // the warp's last read of this tile
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&acc_empty[team]);
+                }
+                long long Z[8];
+#pragma unroll
+                for (int j = 0; j < 8; ++j)
+                    Z[j] = fixed_add(0, __uint_as_float(r0[j]), __uint_as_float(r1[j]),
+                                     g.s > 2 ? __uint_as_float(r2[j]) : 0.0f);
+                emit8(g, Z, ea, m, n0 + b * 8, crow, lane);
+            }
+            if (grp >= NB8) {  // fewer blocks than warps: this one read nothing
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&acc_empty[team]);
+            }
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 0) {
+        tc_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS) : "memory");
+    }
+}
+
+// split-K partials -> C: an exact int64 sum (|Z| < 2^59 at 16384 of K, so up to
+// K = 2^17 in all), in FP64 beyond
+constexpr int COMBINE_INT64_K = 1 << 17;
+__global__ void k_oz_combine(const long long* __restrict__ PZ, int splits, int wide, int Mpad, int Npad, int M, int N,
+                             const int* __restrict__ eA, const int* __restrict__ eB, double alpha, double beta,
+                             double* __restrict__ C, View out_r, View out_c) {
+    const size_t total = (size_t)M * N, zs = (size_t)Mpad * Npad;
     for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < total; t += (size_t)gridDim.x * blockDim.x) {
         const int m = (int)(t / N), n = (int)(t % N);
-        // split-K runs only for small outputs: FP64 sums here are cheap and
-        // cannot overflow however many splits there are
-        double v = 0.0;
-        for (int z = 0; z < splits; ++z) {
-            const size_t idx = ((size_t)z * Mpad + m) * Npad + n;
-            const long long T = (long long)PS0[idx] * 256 + (long long)PS1[idx];
-            v += (double)T + (double)(PF[idx] * 256.0f);
+        const long long* p = PZ + (size_t)m * Npad + n;
+        const int e = safe_exp(eA[m]) + safe_exp(eB[n]) - 44;
+        double v;
+        if (!wide) {
+            long long z = 0;
+#pragma unroll 4
+            for (int q = 0; q < splits; ++q) z += p[q * zs];
+            v = z_scaled(z, e);
+        } else {
+            v = 0.0;
+            for (int q = 0; q < splits; ++q) v += (double)p[q * zs];
+            v = e > BAD_EXP / 2 ? __longlong_as_double(0x7ff8000000000000ll) : scale_pow2(v, e);
         }
-        v = (eA[m] > 1024 || eB[n] > 1024) ? __longlong_as_double(0x7ff8000000000000ll)  // non-finite operand
-                                           : scale_pow2(v, eA[m] + eB[n] - 24);
         if (alpha != 1.0) v *= alpha;
         double* cp = C + view_offset32(out_r, (unsigned)m) + view_offset32(out_c, (unsigned)n);
         *cp = (beta == 0.0) ? v : fma(beta, *cp, v);
@@ -1173,59 +1431,93 @@ bool make_map(CUtensorMap* map, const void* slices, int R, int Kp, int s, int bo
 
 struct Plan {
     int nb16, bn, m_tiles, n_tiles, ksplit, kb_per_split, nkb, stages;
+    bool one;  // a single exact chunk: k_oz_gemm_short
     uint32_t a_bytes, stage_bytes;
     size_t smem, ws_bytes;
 };
+
+// An MMA of BN columns takes about 55 + BN/3 cycles here (measured at 64, 96
+// and 144; 128-row operands from shared memory).
+double mma_cycles(int bn) { return 55.0 + bn / 3.0; }
 
 // mode 2 (3xTF32) holds 16 k per 64-byte stage row instead of 32; modes 1 and
 // 2 never split K
 Plan plan_of(int M, int N, int K, int s, int mode = 0) {
     Plan p{};
-    // fewest 144-wide tiles, then the narrowest 16-multiple width that covers N
-    const int nt = (N + 143) / 144;
-    p.nb16 = ((N + nt - 1) / nt + 15) / 16;
-    if (p.nb16 < 1) p.nb16 = 1;
-    p.bn = 16 * p.nb16;
     p.m_tiles = (M + oz::BM - 1) / oz::BM;
-    p.n_tiles = (N + p.bn - 1) / p.bn;
     p.nkb = mode == 2 ? (k4_of(K) + 15) / 16 : (k8_of(K) + oz::BK - 1) / oz::BK;
     if (p.nkb < 1) p.nkb = 1;
+    p.one = mode == 0 && p.nkb <= oz::CHUNK_KB;
+    if (p.one) {
+        // the width with the least work on the fullest SM: a tile costs the longer
+        // of its MMAs and its epilogue (~0.55 cycles per entry and SM, measured)
+        double best = -1.0;
+        for (int nb = 1; nb <= 5; ++nb) {
+            const double nt = std::ceil(N / (16.0 * nb));
+            const double tile = std::max(2.0 * p.nkb * (s * (s + 1) / 2) * mma_cycles(16 * nb), 0.55 * 128 * 16 * nb) + 600.0;
+            const double cost = std::ceil(nt * p.m_tiles / 152.0) * tile;
+            if (best < 0.0 || cost < best) {
+                best = cost;
+                p.nb16 = nb;
+            }
+        }
+    } else {
+        // fewest 144-wide tiles, then the narrowest 16-multiple width that covers N
+        const int nt = (N + 143) / 144;
+        p.nb16 = std::max(1, ((N + nt - 1) / nt + 15) / 16);
+    }
+    p.bn = 16 * p.nb16;
+    p.n_tiles = (N + p.bn - 1) / p.bn;
     const int nchunks = (p.nkb + oz::CHUNK_KB - 1) / oz::CHUNK_KB;
     const int tiles = p.m_tiles * p.n_tiles;
+    // Split K when the tiles leave SMs idle (at any 32 of K: the sums are exact
+    // int64): the split whose fullest SM has the least work, 2 s(s+1)/2 MMAs per
+    // k-block, a drain per chunk, and the partials' pass.  64 tiles x 256
+    // k-blocks in 3 splits put 176 k-blocks on some SMs, in 2 splits 128 on all.
     int ks = 1;
-    if (mode == 0 && tiles < 120 && nchunks >= 2) ks = std::min(nchunks, (148 + tiles - 1) / tiles);
-    // int32 level sums stay exact for K <= 16384 per split
-    const int max_chunks_per_split = 16384 / (oz::CHUNK_KB * oz::BK);
-    if (mode == 0) ks = std::max(ks, (nchunks + max_chunks_per_split - 1) / max_chunks_per_split);
-    const int cps = (nchunks + ks - 1) / ks;
-    p.kb_per_split = mode == 0 ? cps * oz::CHUNK_KB : p.nkb;
+    if (mode == 0 && tiles < 120 && nchunks >= 2) {
+        const double kb = (double)s * (s + 1) * mma_cycles(p.bn);
+        double best = -1.0;
+        for (int k = 2; k <= p.nkb && k <= 256; ++k) {
+            const int per = (p.nkb + k - 1) / k;
+            if ((p.nkb + per - 1) / per != k) continue;
+            const double cta = per * kb + 2500.0 * ((per + oz::CHUNK_KB - 1) / oz::CHUNK_KB) + 5000.0;
+            const double cost = ((tiles * k + 151) / 152) * cta + 8.0 * k * p.m_tiles * oz::BM * p.n_tiles * p.bn / 1500.0;
+            if (best < 0.0 || cost < best) {
+                best = cost;
+                ks = k;
+            }
+        }
+    }
+    // int64 sums of a split stay below 2^59 for K <= 16384
+    const int max_kb_per_split = 16384 / oz::BK;
+    if (mode == 0) ks = std::max(ks, (p.nkb + max_kb_per_split - 1) / max_kb_per_split);
+    p.kb_per_split = mode == 0 ? (p.nkb + ks - 1) / ks : p.nkb;
     p.ksplit = (p.nkb + p.kb_per_split - 1) / p.kb_per_split;
     p.a_bytes = (uint32_t)(s * oz::BM * oz::BK * 2);
     p.stage_bytes = p.a_bytes + (uint32_t)(s * p.bn * oz::BK * 2);
     p.stages = std::min<int>(6, (int)((220u * 1024u) / p.stage_bytes));
     p.smem = (size_t)p.stages * p.stage_bytes + 1024 + 256;
-    p.ws_bytes = p.ksplit > 1 ? 3 * align256((size_t)p.ksplit * p.m_tiles * oz::BM * p.n_tiles * p.bn * 4) : 0;
+    p.ws_bytes = p.ksplit > 1 ? align256((size_t)p.ksplit * p.m_tiles * oz::BM * p.n_tiles * p.bn * 8) : 0;
     return p;
 }
 
-template <int NB16, bool ONE, int MODE = 0>
-cudaError_t launch_gemm(const Plan& p, const CUtensorMap& ta, const CUtensorMap& tb, const oz::GemmArgs& g,
-                        cudaStream_t st) {
-    // the 227 KB dynamic shared-memory opt-in is a per-device function
-    // attribute: set it once for every device this instantiation runs on
+using GemmKernel = void (*)(const CUtensorMap, const CUtensorMap, const oz::GemmArgs);
+// `done`: a bit per device on which this kernel's 227 KB shared-memory opt-in
+// (a per-device function attribute) is set
+cudaError_t launch_gemm(GemmKernel kern, int threads, unsigned long long* done, const Plan& p, const CUtensorMap& ta,
+                        const CUtensorMap& tb, const oz::GemmArgs& g, cudaStream_t st) {
     static std::mutex mu;
-    static unsigned long long done = 0;  // bit per device
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
     {
         std::lock_guard<std::mutex> lock(mu);
-        if (!(done >> dev & 1ull)) {
-            e = cudaFuncSetAttribute(oz::k_oz_gemm<NB16, ONE, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     227 * 1024);
+        if (!(*done >> dev & 1ull)) {
+            e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
             if (e != cudaSuccess) return e;
-            done |= 1ull << dev;
+            *done |= 1ull << dev;
         }
     }
     dim3 grid(p.m_tiles, p.n_tiles, p.ksplit);
@@ -1238,8 +1530,18 @@ cudaError_t launch_gemm(const Plan& p, const CUtensorMap& ta, const CUtensorMap&
         grid = dim3((unsigned)std::min<long long>(tiles, nsm > 0 ? nsm : 1), 1, 1);
     }
     ++g_launches;
-    oz::k_oz_gemm<NB16, ONE, MODE><<<grid, oz::THREADS, p.smem, st>>>(ta, tb, g);
+    kern<<<grid, threads, p.smem, st>>>(ta, tb, g);
     return cudaGetLastError();
+}
+template <int NB16>
+cudaError_t launch_mode(int mode, const Plan& p, const CUtensorMap& ta, const CUtensorMap& tb, const oz::GemmArgs& g,
+                        cudaStream_t st) {
+    static unsigned long long done[4] = {};
+    if constexpr (NB16 <= 5)
+        if (p.one) return launch_gemm(oz::k_oz_gemm_short<NB16>, oz::SHORT_THREADS, done + 3, p, ta, tb, g, st);
+    if (mode == 0) return launch_gemm(oz::k_oz_gemm<NB16, 0>, oz::THREADS, done, p, ta, tb, g, st);
+    if (mode == 1) return launch_gemm(oz::k_oz_gemm<NB16, 1>, oz::THREADS, done + 1, p, ta, tb, g, st);
+    return launch_gemm(oz::k_oz_gemm<NB16, 2>, oz::THREADS, done + 2, p, ta, tb, g, st);
 }
 
 }  // namespace
@@ -1436,70 +1738,47 @@ cudaError_t oz_gemm_view(int M, int N, int K, int s, const void* Asplit, const v
         g.out_c.dim[a] = ocv.dim[a];
         g.out_c.stride[a] = ocv.stride[a];
     }
+    // Output columns that lie together are stored 32 or 16 bytes at a time: a
+    // lane holds a row, and 8-byte stores to 32 rows left every sector written
+    // in four parts (262144 x 192 x 64, row-major: 415 us).  Groups of `vec`
+    // columns must be contiguous and aligned for every row.
+    g.plain = alpha == 1.0 && beta == 0.0;
+    g.vec = 1;
+    if (g.plain)
+        for (int v : {4, 2}) {
+            bool ok = (uintptr_t)C % (8 * v) == 0 && ocv.stride[ocv.n - 1] == 1 && (ocv.n == 1 || ocv.dim[ocv.n - 1] % v == 0);
+            for (int a = 0; a < ocv.n - 1; ++a) ok = ok && ocv.stride[a] % v == 0;
+            for (int a = 0; a < orv.n; ++a) ok = ok && (orv.dim[a] == 1 || orv.stride[a] % v == 0);
+            if (ok) {
+                g.vec = v;
+                break;
+            }
+        }
     g.Mpad = p.m_tiles * oz::BM;
     g.m_tiles = p.m_tiles;
     g.n_tiles = p.n_tiles;
     g.Npad = p.n_tiles * p.bn;
-    if (!g.direct) {
-        const size_t part = align256((size_t)p.ksplit * g.Mpad * g.Npad * 4);
-        g.PS0 = (int*)ws;
-        g.PS1 = (int*)((char*)ws + part);
-        g.PF = (float*)((char*)ws + 2 * part);
-    }
+    if (!g.direct) g.PZ = (long long*)ws;
     g.err = err;
     g.wait_limit = oz::WAIT_LIMIT_CYCLES;
-    // a CTA's K range: all of K (direct) or kb_per_split k-blocks (split-K)
-    const bool one = (p.ksplit == 1 ? p.nkb : p.kb_per_split) <= oz::CHUNK_KB;
     cudaError_t e;
-    if (mode != 0) {
-        switch (p.nb16 * 4 + mode) {
-            case 5: e = launch_gemm<1, true, 1>(p, ta, tb, g, st); break;
-            case 6: e = launch_gemm<1, true, 2>(p, ta, tb, g, st); break;
-            case 9: e = launch_gemm<2, true, 1>(p, ta, tb, g, st); break;
-            case 10: e = launch_gemm<2, true, 2>(p, ta, tb, g, st); break;
-            case 13: e = launch_gemm<3, true, 1>(p, ta, tb, g, st); break;
-            case 14: e = launch_gemm<3, true, 2>(p, ta, tb, g, st); break;
-            case 17: e = launch_gemm<4, true, 1>(p, ta, tb, g, st); break;
-            case 18: e = launch_gemm<4, true, 2>(p, ta, tb, g, st); break;
-            case 21: e = launch_gemm<5, true, 1>(p, ta, tb, g, st); break;
-            case 22: e = launch_gemm<5, true, 2>(p, ta, tb, g, st); break;
-            case 25: e = launch_gemm<6, true, 1>(p, ta, tb, g, st); break;
-            case 26: e = launch_gemm<6, true, 2>(p, ta, tb, g, st); break;
-            case 29: e = launch_gemm<7, true, 1>(p, ta, tb, g, st); break;
-            case 30: e = launch_gemm<7, true, 2>(p, ta, tb, g, st); break;
-            case 33: e = launch_gemm<8, true, 1>(p, ta, tb, g, st); break;
-            case 34: e = launch_gemm<8, true, 2>(p, ta, tb, g, st); break;
-            case 37: e = launch_gemm<9, true, 1>(p, ta, tb, g, st); break;
-            default: e = launch_gemm<9, true, 2>(p, ta, tb, g, st); break;
-        }
-        return e;
-    }
-    switch (p.nb16 * 2 + (one ? 1 : 0)) {
-        case 2: e = launch_gemm<1, false>(p, ta, tb, g, st); break;
-        case 3: e = launch_gemm<1, true>(p, ta, tb, g, st); break;
-        case 4: e = launch_gemm<2, false>(p, ta, tb, g, st); break;
-        case 5: e = launch_gemm<2, true>(p, ta, tb, g, st); break;
-        case 6: e = launch_gemm<3, false>(p, ta, tb, g, st); break;
-        case 7: e = launch_gemm<3, true>(p, ta, tb, g, st); break;
-        case 8: e = launch_gemm<4, false>(p, ta, tb, g, st); break;
-        case 9: e = launch_gemm<4, true>(p, ta, tb, g, st); break;
-        case 10: e = launch_gemm<5, false>(p, ta, tb, g, st); break;
-        case 11: e = launch_gemm<5, true>(p, ta, tb, g, st); break;
-        case 12: e = launch_gemm<6, false>(p, ta, tb, g, st); break;
-        case 13: e = launch_gemm<6, true>(p, ta, tb, g, st); break;
-        case 14: e = launch_gemm<7, false>(p, ta, tb, g, st); break;
-        case 15: e = launch_gemm<7, true>(p, ta, tb, g, st); break;
-        case 16: e = launch_gemm<8, false>(p, ta, tb, g, st); break;
-        case 17: e = launch_gemm<8, true>(p, ta, tb, g, st); break;
-        case 18: e = launch_gemm<9, false>(p, ta, tb, g, st); break;
-        default: e = launch_gemm<9, true>(p, ta, tb, g, st); break;
+    switch (p.nb16) {
+        case 1: e = launch_mode<1>(mode, p, ta, tb, g, st); break;
+        case 2: e = launch_mode<2>(mode, p, ta, tb, g, st); break;
+        case 3: e = launch_mode<3>(mode, p, ta, tb, g, st); break;
+        case 4: e = launch_mode<4>(mode, p, ta, tb, g, st); break;
+        case 5: e = launch_mode<5>(mode, p, ta, tb, g, st); break;
+        case 6: e = launch_mode<6>(mode, p, ta, tb, g, st); break;
+        case 7: e = launch_mode<7>(mode, p, ta, tb, g, st); break;
+        case 8: e = launch_mode<8>(mode, p, ta, tb, g, st); break;
+        default: e = launch_mode<9>(mode, p, ta, tb, g, st); break;
     }
     if (e != cudaSuccess || g.direct) return e;
     size_t blocks = ((size_t)M * N + 255) / 256;
     if (blocks > 152 * 16) blocks = 152 * 16;
     ++g_launches;
-    oz::k_oz_combine<<<(unsigned)blocks, 256, 0, st>>>(g.PS0, g.PS1, g.PF, p.ksplit, g.Mpad, g.Npad, M, N, g.eA,
-                                                        g.eB, alpha, beta, C, g.out_r, g.out_c);
+    oz::k_oz_combine<<<(unsigned)blocks, 256, 0, st>>>(g.PZ, p.ksplit, K > oz::COMBINE_INT64_K ? 1 : 0, g.Mpad, g.Npad,
+                                                        M, N, g.eA, g.eB, alpha, beta, C, g.out_r, g.out_c);
     return cudaGetLastError();
 }
 
