@@ -83,6 +83,13 @@ struct ctm_ctx {
     // scratch
     double *X1 = nullptr, *S1 = nullptr, *S2 = nullptr, *S3 = nullptr;
     double* E[8] = {};        // ul, ur, br, bl of the current cut (E[4..7]: the second cut when batched)
+    // enlarged corners a sweep keeps for its next steps (batch_cuts): the
+    // buffers the E above are drawn from, and which corner (site, position)
+    // each holds, -1 when none; valid within one sweep only
+    static constexpr int NEB = 12;
+    double* Eb[NEB] = {};
+    int eb_corner[NEB];
+    int n_eb = 0;
     // second cut's range-finder bases and SVD factors (batch_cuts)
     double *Qm1 = nullptr, *Qb1 = nullptr, *G1 = nullptr, *Us1 = nullptr, *Ws1 = nullptr, *Sv1 = nullptr;
     void* svd2_ws = nullptr;
@@ -371,11 +378,27 @@ void slices_written(ctm_ctx* h, const double* p) {
     for (auto& c : h->ozc)
         if (c.ptr == p) c.valid = false;
 }
+// the slice cache of a resident corner A (plain or transposed): the one that
+// holds it, else one that holds nothing valid, else one of a corner that the
+// current cuts do not use (two caches per current corner exist)
 int slice_slot(ctm_ctx* h, const double* A, bool tA, int M, int K) {
-    if (!h->ozc[0].buf || M != h->N || K != h->N) return -1;
-    for (int c = 0; c < 8; ++c)
-        if (A && A == h->E[c]) return 2 * c + (tA ? 1 : 0);
-    return -1;
+    if (!h->ozc[0].buf || M != h->N || K != h->N || !A) return -1;
+    auto current = [&](const double* p) { return std::find(h->E, h->E + 8, p) != h->E + 8; };
+    if (!current(A)) return -1;
+    int idle = -1, other = -1;
+    for (int c = 0; c < 16 && h->ozc[c].buf; ++c) {
+        const auto& o = h->ozc[c];
+        if (o.ptr == A && o.trans == tA) return c;
+        if (!o.valid && idle < 0) idle = c;
+        if (!current(o.ptr) && other < 0) other = c;
+    }
+    const int c = idle >= 0 ? idle : other;
+    if (c >= 0) {
+        h->ozc[c].ptr = A;
+        h->ozc[c].trans = tA;
+        h->ozc[c].valid = false;
+    }
+    return c;
 }
 // operand slices of the handle's scheme for an R x K operand on strided views
 ctm_status split_v(ctm_ctx* h, const double* X, int R, int K, const OzView& rv, const OzView& kv, void* dst) {
@@ -655,6 +678,52 @@ ctm_status svd2_(ctm_ctx* h, const CutBufs& a, const CutBufs& b) {
     return CTM_OK;
 }
 
+// Corners of a column step out of those the sweep already holds.  Corner c of
+// a site is made of C_c, T_c, T_{c-1}; a move m rewrites C_m, C_{m+3} and
+// T_{m+3} of the next column's sites only, so its right-hand corners (c = m+1,
+// m+2, of all four sites after its two steps) stay what they are: the next
+// move takes the former as its upper-left corners (in its first step, before
+// it rewrites them) and the latter as its upper-right ones.  46 of a sweep's
+// 64 corners are computed; at most eight are kept beside the four of a step
+// that are new.
+int corner_id(int site, int c) { return 4 * site + (c & 3); }
+// E[r], r < 8, for the corners ids[r]: resident ones by pointer, the others
+// computed into buffers that hold none of `keep` (a predicate) or of ids
+template <class Keep>
+ctm_status resident_corners(ctm_ctx* h, const int* ids, Keep keep) {
+    bool taken[ctm_ctx::NEB] = {};
+    int at[8];
+    for (int r = 0; r < 8; ++r) {
+        at[r] = -1;
+        for (int b = 0; b < h->n_eb; ++b)
+            if (h->eb_corner[b] == ids[r]) at[r] = b;
+        if (at[r] >= 0) taken[at[r]] = true;
+    }
+    for (int b = 0; b < h->n_eb; ++b)
+        if (h->eb_corner[b] >= 0 && keep(h->eb_corner[b])) taken[b] = true;
+    bool fresh[8] = {};
+    for (int r = 0; r < 8; ++r) {
+        if (at[r] < 0) {
+            int b = 0;
+            while (b < h->n_eb && taken[b]) ++b;
+            if (b == h->n_eb) {
+                h->err = "no buffer for an enlarged corner";
+                return CTM_ERR_STATE;
+            }
+            taken[b] = true;
+            fresh[r] = true;
+            at[r] = b;
+        }
+        h->E[r] = h->Eb[at[r]];
+    }
+    for (int r = 0; r < 8; ++r)
+        if (fresh[r]) {
+            h->eb_corner[at[r]] = ids[r];
+            CKS(enlarged_corner(h, ids[r] / 4, ids[r] & 3, h->E[r]));
+        }
+    return CTM_OK;
+}
+
 ctm_status normalise_into(ctm_ctx* h, const double* src, double* dst, size_t n, int slot) {
     CK(cudaMemsetAsync(h->maxbits + slot, 0, sizeof(unsigned long long), h->stream));
     CK(ctm::maxabs(src, n, h->maxbits + slot, h->stream));
@@ -667,23 +736,40 @@ ctm_status normalise_into(ctm_ctx* h, const double* src, double* dst, size_t n, 
 ctm_status left_move(ctm_ctx* h, int m, int x) {
     const int chi = h->chi, N = h->N, D = h->D;
     const bool both = h->E[4] != nullptr;  // batch_cuts: corners of both cuts resident
+    if (both) {
+        int ids[8];
+        for (int y = 0; y < 2; ++y) {
+            ids[4 * y + 0] = corner_id(FM.site(m, x, y + 1), m + 0);
+            ids[4 * y + 1] = corner_id(FM.site(m, x + 1, y + 1), m + 1);
+            ids[4 * y + 2] = corner_id(FM.site(m, x + 1, y), m + 2);
+            ids[4 * y + 3] = corner_id(FM.site(m, x, y), m + 3);
+        }
+        const int c1 = (m + 1) & 3, c2 = (m + 2) & 3;
+        CKS(resident_corners(h, ids, [&](int id) { return h->n_eb > 8 && ((id & 3) == c1 || (id & 3) == c2); }));
+    }
     for (int y = 0; y < 2; ++y) {
+        const int cut = ((m & 3) * 2 + x) * 2 + y;
+        if (both) {
+            CKS(range_finder(h, cut, cut_bufs(h, y)));
+            continue;
+        }
         const int tl = FM.site(m, x, y + 1), tr = FM.site(m, x + 1, y + 1);
         const int br = FM.site(m, x + 1, y), bl = FM.site(m, x, y);
-        double* const* E = both ? h->E + 4 * y : h->E;
-        CKS(enlarged_corner(h, tl, m + 0, E[0]));
-        CKS(enlarged_corner(h, tr, m + 1, E[1]));
-        CKS(enlarged_corner(h, br, m + 2, E[2]));
-        CKS(enlarged_corner(h, bl, m + 3, E[3]));
-        const int cut = ((m & 3) * 2 + x) * 2 + y;
-        if (!both) CKS(projectors(h, y, cut));
-        else CKS(range_finder(h, cut, cut_bufs(h, y)));
+        CKS(enlarged_corner(h, tl, m + 0, h->E[0]));
+        CKS(enlarged_corner(h, tr, m + 1, h->E[1]));
+        CKS(enlarged_corner(h, br, m + 2, h->E[2]));
+        CKS(enlarged_corner(h, bl, m + 3, h->E[3]));
+        CKS(projectors(h, y, cut));
     }
     if (both) {
         CKS(svd2_(h, cut_bufs(h, 0), cut_bufs(h, 1)));
         for (int y = 0; y < 2; ++y) CKS(finish_projectors(h, y, ((m & 3) * 2 + x) * 2 + y, cut_bufs(h, y)));
     }
     ProfTag tg(h, "absorb");
+    // the upper-left corner of the first cut is not needed any more: its buffer
+    // is the absorption's scratch
+    for (int b = 0; b < h->n_eb; ++b)
+        if (h->Eb[b] == h->E[0]) h->eb_corner[b] = -1;
     for (int y = 0; y < 2; ++y) {
         const int i = FM.site(m, x, y), j = FM.site(m, x + 1, y);
         const int ym = (y + 1) % 2;  // cut between rows y-1 and y
@@ -703,14 +789,22 @@ ctm_status left_move(ctm_ctx* h, int m, int x) {
         CKS(normalise_into(h, h->newC1, ej[Cw(m)], (size_t)chi * chi, 0));
         CKS(normalise_into(h, h->newT4, ej[Tw(m + 3)], (size_t)chi * N, 1));
         CKS(normalise_into(h, h->newC4, ej[Cw(m + 3)], (size_t)chi * chi, 2));
+        for (int b = 0; b < h->n_eb; ++b)
+            if (h->eb_corner[b] == corner_id(j, m) || h->eb_corner[b] == corner_id(j, m + 3)) h->eb_corner[b] = -1;
     }
     return CTM_OK;
 }
 
 ctm_status one_sweep_eager(ctm_ctx* h) {
-    for (int m = 0; m < 4; ++m)
-        for (int x = 0; x < 2; ++x) CKS(left_move(h, m, x));
-    return CTM_OK;
+    // other calls use the corners' buffers (and S3) as scratch: a sweep starts
+    // with none of its corners, and leaves E on its own buffers
+    std::fill(h->eb_corner, h->eb_corner + ctm_ctx::NEB, -1);
+    ctm_status st = CTM_OK;
+    for (int m = 0; m < 4 && st == CTM_OK; ++m)
+        for (int x = 0; x < 2 && st == CTM_OK; ++x) st = left_move(h, m, x);
+    if (h->n_eb)
+        for (int r = 0; r < 8; ++r) h->E[r] = h->Eb[r];
+    return st;
 }
 
 // A sweep's launch sequence is fixed once every cut has a warm basis (or
@@ -1444,6 +1538,16 @@ ctm_status create(int Lx, int Ly, int d, int D, const ctm_options* o, void* stre
     A_(&h->S3, z.open);
     A_(&h->S2, (size_t)d * z.NN);
     for (int c = 0; c < (o->batch_cuts ? 8 : 4); ++c) A_(&h->E[c], z.NN);
+    if (o->batch_cuts && st == CTM_OK) {
+        for (int c = 0; c < 8; ++c) h->Eb[c] = h->E[c];
+        h->n_eb = 8;
+        // S3 serves the density matrices' open corners only (d^2 N^2): a sweep
+        // keeps four more corners there
+        if (d >= 2) {
+            for (int c = 0; c < 4; ++c) h->Eb[8 + c] = h->S3 + c * z.NN;
+            h->n_eb = 12;
+        }
+    }
     if (o->batch_cuts) {
         A_(&h->Qm1, z.Nk); A_(&h->Qb1, z.Nk); A_(&h->G1, z.kk); A_(&h->Us1, z.kk); A_(&h->Ws1, z.kk);
         A_(&h->Sv1, h->k);
