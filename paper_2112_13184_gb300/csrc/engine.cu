@@ -101,6 +101,19 @@ struct ctm_ctx {
     double *Lh = nullptr, *Rh = nullptr, *rho = nullptr, *spec = nullptr, *corners = nullptr;
     double* splitk = nullptr;  // split-K partial sums
     size_t splitk_n = 0;
+    // Second branch of a column step (small handles): the two cuts' range
+    // finders, and their projectors, run side by side on two streams.  The
+    // scratch of the second; BranchScope exchanges it with the fields above
+    // and below while that branch's calls are issued.
+    struct Branch {
+        cudaStream_t stream = nullptr;
+        double *Om = nullptr, *Yb = nullptr, *Zb = nullptr, *Qm2 = nullptr, *Rb = nullptr, *Uc = nullptr, *Vc = nullptr;
+        double *t1 = nullptr, *t2 = nullptr, *inv = nullptr, *splitk = nullptr;
+        size_t splitk_n = 0, ozA_n = 0, ozB_n = 0, ozW_n = 0;
+        void *ozA = nullptr, *ozB = nullptr, *ozW = nullptr, *qr_ws = nullptr;
+    } br;
+    bool fork = false;
+    cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
     // emulated-FP64 tensor-core GEMMs: operand slices and split-K partials
     void *ozA = nullptr, *ozB = nullptr, *ozW = nullptr;
     size_t ozA_n = 0, ozB_n = 0, ozW_n = 0;
@@ -225,6 +238,33 @@ OzBounds oz_bounds(int d, int D, int chi, int k, int s, int mode) {
         z.a = std::max(z.a, tc_split_bytes((int)sh[0], (int)sh[2], mode, s));
         z.b = std::max(z.b, tc_split_bytes((int)sh[1], (int)sh[2], mode, s));
         z.w = std::max(z.w, ctm::oz_gemm_ws_bytes((int)sh[0], (int)sh[1], (int)sh[2], s, mode));
+    }
+    return z;
+}
+
+// The two cuts of a column step side by side: worth it where one cut leaves
+// most of the chip idle, i.e. where its QR runs in one 16-CTA cluster.  (At
+// d=2, D=4, chi=32 a column step is ~250 kernels of a few microseconds on a
+// tenth of the SMs; at D=6, chi=48 and above each kernel fills them.)
+bool forks(int N, int k, const ctm_options& o) { return o.batch_cuts && ctm::qr_one_cluster(N, k); }
+struct BranchSizes {
+    size_t Nk, kk, tk, splitk, ozA = 0, ozB = 0, ozW = 0;
+};
+BranchSizes branch_sizes(int N, int chi, int k, const ctm_options& o) {
+    BranchSizes z;
+    z.Nk = (size_t)N * k;
+    z.kk = (size_t)k * k;
+    z.tk = (size_t)N * std::max(k, chi);
+    z.splitk = 32 * z.tk;
+    const int mode = tc_mode_of(o.precision), s = tc_slices_of(o);
+    if (mode >= 0) {
+        const int shapes[4][3] = {{N, k, N}, {N, chi, N}, {N, chi, k}, {N, k, k}};
+        for (const auto& h : shapes) {
+            z.ozA = std::max(z.ozA, tc_split_bytes(h[0], h[2], mode, s));
+            z.ozB = std::max(z.ozB, tc_split_bytes(h[1], h[2], mode, s));
+            z.ozW = std::max(z.ozW, ctm::oz_gemm_ws_bytes(h[0], h[1], h[2], s, mode));
+        }
+        z.ozW = std::max<size_t>(z.ozW, 256);
     }
     return z;
 }
@@ -669,6 +709,59 @@ ctm_status projectors(ctm_ctx* h, int slot, int cut) {
     return finish_projectors(h, slot, cut, c);
 }
 
+// While it lives, the handle's calls go to the second branch's stream with
+// its scratch: opened after what the branch needs is enqueued on the handle's
+// stream, and followed by join_branch before anything that needs its results.
+struct BranchScope {
+    ctm_ctx* h;
+    explicit BranchScope(ctm_ctx* h_) : h(h_) { exchange(); }
+    ~BranchScope() { exchange(); }
+    BranchScope(const BranchScope&) = delete;
+    void exchange() {
+        auto& b = h->br;
+        std::swap(h->stream, b.stream);
+        std::swap(h->Om, b.Om);
+        std::swap(h->Yb, b.Yb);
+        std::swap(h->Zb, b.Zb);
+        std::swap(h->Qm2, b.Qm2);
+        std::swap(h->Rb, b.Rb);
+        std::swap(h->Uc, b.Uc);
+        std::swap(h->Vc, b.Vc);
+        std::swap(h->t1, b.t1);
+        std::swap(h->t2, b.t2);
+        std::swap(h->inv, b.inv);
+        std::swap(h->splitk, b.splitk);
+        std::swap(h->splitk_n, b.splitk_n);
+        std::swap(h->ozA, b.ozA);
+        std::swap(h->ozB, b.ozB);
+        std::swap(h->ozW, b.ozW);
+        std::swap(h->ozA_n, b.ozA_n);
+        std::swap(h->ozB_n, b.ozB_n);
+        std::swap(h->ozW_n, b.ozW_n);
+        std::swap(h->qr_ws, b.qr_ws);
+    }
+};
+// f(0) on the handle's stream beside f(1) on the second branch, or one after
+// the other.  Whatever fails, the branch is joined: nothing of it may be left
+// running (or uncaptured) behind the handle's stream.
+template <class F>
+ctm_status both_cuts(ctm_ctx* h, F f) {
+    if (!h->fork || h->prof) {
+        CKS(f(0));
+        return f(1);
+    }
+    CK(cudaEventRecord(h->ev_fork, h->stream));
+    CK(cudaStreamWaitEvent(h->br.stream, h->ev_fork, 0));
+    ctm_status st = f(0);  // first, as without branches: the random test matrices are drawn in this order
+    if (st == CTM_OK) {
+        BranchScope scope(h);
+        st = f(1);
+    }
+    CK(cudaEventRecord(h->ev_join, h->br.stream));
+    CK(cudaStreamWaitEvent(h->stream, h->ev_join, 0));
+    return st;
+}
+
 // both cuts' SVDs in one launch (two Jacobi clusters)
 ctm_status svd2_(ctm_ctx* h, const CutBufs& a, const CutBufs& b) {
     ProfTag tg(h, "svd");
@@ -747,23 +840,21 @@ ctm_status left_move(ctm_ctx* h, int m, int x) {
         const int c1 = (m + 1) & 3, c2 = (m + 2) & 3;
         CKS(resident_corners(h, ids, [&](int id) { return h->n_eb > 8 && ((id & 3) == c1 || (id & 3) == c2); }));
     }
-    for (int y = 0; y < 2; ++y) {
-        const int cut = ((m & 3) * 2 + x) * 2 + y;
-        if (both) {
-            CKS(range_finder(h, cut, cut_bufs(h, y)));
-            continue;
-        }
-        const int tl = FM.site(m, x, y + 1), tr = FM.site(m, x + 1, y + 1);
-        const int br = FM.site(m, x + 1, y), bl = FM.site(m, x, y);
-        CKS(enlarged_corner(h, tl, m + 0, h->E[0]));
-        CKS(enlarged_corner(h, tr, m + 1, h->E[1]));
-        CKS(enlarged_corner(h, br, m + 2, h->E[2]));
-        CKS(enlarged_corner(h, bl, m + 3, h->E[3]));
-        CKS(projectors(h, y, cut));
-    }
+    auto cut_of = [&](int y) { return ((m & 3) * 2 + x) * 2 + y; };
     if (both) {
+        CKS(both_cuts(h, [&](int y) { return range_finder(h, cut_of(y), cut_bufs(h, y)); }));
         CKS(svd2_(h, cut_bufs(h, 0), cut_bufs(h, 1)));
-        for (int y = 0; y < 2; ++y) CKS(finish_projectors(h, y, ((m & 3) * 2 + x) * 2 + y, cut_bufs(h, y)));
+        CKS(both_cuts(h, [&](int y) { return finish_projectors(h, y, cut_of(y), cut_bufs(h, y)); }));
+    } else {
+        for (int y = 0; y < 2; ++y) {
+            const int tl = FM.site(m, x, y + 1), tr = FM.site(m, x + 1, y + 1);
+            const int br = FM.site(m, x + 1, y), bl = FM.site(m, x, y);
+            CKS(enlarged_corner(h, tl, m + 0, h->E[0]));
+            CKS(enlarged_corner(h, tr, m + 1, h->E[1]));
+            CKS(enlarged_corner(h, br, m + 2, h->E[2]));
+            CKS(enlarged_corner(h, bl, m + 3, h->E[3]));
+            CKS(projectors(h, y, cut_of(y)));
+        }
     }
     ProfTag tg(h, "absorb");
     // the upper-left corner of the first cut is not needed any more: its buffer
@@ -1564,6 +1655,40 @@ ctm_status create(int Lx, int Ly, int d, int D, const ctm_options* o, void* stre
     A_(&h->rho, std::max<size_t>(64 * 64, (size_t)d * d * d * d));
     h->splitk_n = (size_t)1 << 24;
     A_(&h->splitk, h->splitk_n);
+    if (st == CTM_OK && forks(h->N, h->k, *o)) {
+        // the second branch's scratch is the tail of the split-K partials' buffer,
+        // which no product of a handle this small fills
+        const BranchSizes b = branch_sizes(h->N, h->chi, h->k, *o);
+        auto& r = h->br;
+        size_t used = 0;
+        auto take = [&](size_t bytes) {
+            char* p = (char*)h->splitk + used;
+            used += (bytes + 255) & ~(size_t)255;
+            return (void*)p;
+        };
+        auto dbl = [&](size_t n) { return (double*)take(n * sizeof(double)); };
+        double* const whole = h->splitk;
+        r.Om = dbl(b.Nk), r.Yb = dbl(b.Nk), r.Zb = dbl(b.Nk), r.Qm2 = dbl(b.Nk), r.Vc = dbl(b.Nk), r.Rb = dbl(b.kk);
+        r.Uc = dbl(b.tk), r.t1 = dbl(b.tk), r.t2 = dbl(b.tk), r.inv = dbl(h->k), r.splitk = dbl(b.splitk);
+        r.splitk_n = b.splitk;
+        r.qr_ws = take(qr_ws_bytes(h->N, h->k));
+        if (tc_mode_of(o->precision) >= 0) {
+            r.ozA = take(r.ozA_n = b.ozA);
+            r.ozB = take(r.ozB_n = b.ozB);
+            r.ozW = take(r.ozW_n = b.ozW);
+        }
+        if (used <= h->splitk_n * sizeof(double) / 2) {
+            h->splitk = whole + used / sizeof(double);
+            h->splitk_n -= used / sizeof(double);
+            if (cudaStreamCreateWithFlags(&r.stream, cudaStreamNonBlocking) != cudaSuccess ||
+                cudaEventCreateWithFlags(&h->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
+                cudaEventCreateWithFlags(&h->ev_join, cudaEventDisableTiming) != cudaSuccess) {
+                h->err = "cudaStreamCreate failed";
+                st = CTM_ERR_CUDA;
+            }
+            h->fork = st == CTM_OK;
+        }
+    }
     A_(&h->spec, 16 * (size_t)h->chi);
     A_(&h->corners, 16 * z.C);
     if (st == CTM_OK) st = alloc(h, &h->qr_ws, qr_ws_bytes(h->N, h->k));
@@ -1613,6 +1738,9 @@ ctm_status ctm_destroy(ctm_handle h) {
     if (h->graph) cudaGraphDestroy(h->graph);
     for (void* p : h->allocs) cudaFree(p);
     for (cudaEvent_t e : h->ev_pool) cudaEventDestroy(e);
+    if (h->ev_fork) cudaEventDestroy(h->ev_fork);
+    if (h->ev_join) cudaEventDestroy(h->ev_join);
+    if (h->br.stream) cudaStreamDestroy(h->br.stream);  // its work is joined to h->stream, synchronised above
     if (h->own_stream && h->stream) cudaStreamDestroy(h->stream);
     delete h;
     return CTM_OK;

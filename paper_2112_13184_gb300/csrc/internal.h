@@ -53,6 +53,8 @@ size_t qr_ws_bytes(int N, int k);
 // -- or, without err, the first int of ws -- becomes 1 and Q, R are not
 // valid), else two launches per column step.
 cudaError_t qr(const double* Y, int N, int k, double* Q, double* R, void* ws, cudaStream_t s, int* err = nullptr);
+// whether an N x k QR is better off in one 16-CTA cluster than on every SM
+bool qr_one_cluster(int N, int k);
 size_t svd_ws_bytes(int k);
 // *status (optional; else the first int of ws) becomes 1 when the Jacobi
 // iteration still rotated in its last allowed sweep

@@ -788,22 +788,33 @@ __device__ __forceinline__ bool elect_one() {
     asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
     return p != 0;
 }
-// tc_mma on descriptors given by their low words (address, leading offset)
+// tc_mma on descriptors given by their low words (address, leading offset).
+// USE: what becomes of the A operand in the collector buffer -- 0 as it
+// comes, 1 kept for the next MMAs, 2 taken from there and kept, 3 taken from
+// there for the last time.
+template <int USE>
 __device__ __forceinline__ void tc_mma_lo(uint32_t d_tmem, uint32_t alo, uint32_t blo, uint32_t hi, uint32_t idesc,
                                           uint32_t accumulate) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\t"
-        "mov.b64 da, {%1, %3};\n\tmov.b64 db, {%2, %3};\n\t"
-        "setp.ne.b32 p, %5, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, p;\n\t}" ::"r"(d_tmem),
-        "r"(alo), "r"(blo), "r"(hi), "r"(idesc), "r"(accumulate)
-        : "memory");
+#define CTM_MMA_LO(COLLECTOR)                                                                        \
+    asm volatile(                                                                                    \
+        "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\t"                                                \
+        "mov.b64 da, {%1, %3};\n\tmov.b64 db, {%2, %3};\n\t"                                         \
+        "setp.ne.b32 p, %5, 0;\n\t"                                                                  \
+        "tcgen05.mma.cta_group::1.kind::f16" COLLECTOR " [%0], da, db, %4, p;\n\t}" ::"r"(d_tmem),   \
+        "r"(alo), "r"(blo), "r"(hi), "r"(idesc), "r"(accumulate)                                     \
+        : "memory")
+    if (USE == 0) CTM_MMA_LO("");
+    else if (USE == 1) CTM_MMA_LO(".collector::a::fill");
+    else if (USE == 2) CTM_MMA_LO(".collector::a::use");
+    else CTM_MMA_LO(".collector::a::lastuse");
+#undef CTM_MMA_LO
 }
 // All slice products of one 32-wide k-block, S slices: level 0 and level 1 into
 // their accumulators, the rest into the third; keep = 0 restarts the three.
 // Straight-line code on constant offsets from the two tile addresses: issued
 // from loops over runtime slice indices an MMA took 137 cycles whatever its
-// width, so ~100 at N = 144 and 75 at N = 64.
+// width, so ~100 at N = 144 and 75 at N = 64.  A slice by A slice, so that the
+// 128-row operand is read once for its products instead of once for each.
 template <int S, int BN>
 __device__ __forceinline__ void issue_levels(uint32_t tmem, uint32_t sa, uint32_t sb, uint32_t idesc, uint32_t keep) {
     constexpr uint64_t top = (uint64_t)(512 >> 4) << 32 | (uint64_t)1 << 46 | (uint64_t)4 << 61;  // as sw64_desc
@@ -812,15 +823,21 @@ __device__ __forceinline__ void issue_levels(uint32_t tmem, uint32_t sa, uint32_
 #pragma unroll
     for (int h = 0; h < 2; ++h) {  // two K=16 halves, 32 bytes apart in the 64-byte row
         const uint32_t k0 = h ? 1u : keep;
-        tc_mma_lo(tmem, a0 + 2 * h, b0 + 2 * h, hi, idesc, k0);
-        tc_mma_lo(tmem + BN, a0 + 2 * h, b0 + BN * 4 + 2 * h, hi, idesc, k0);
-        tc_mma_lo(tmem + BN, a0 + BM * 4 + 2 * h, b0 + 2 * h, hi, idesc, 1u);
 #pragma unroll
-        for (int L = 2; L < S; ++L)
+        for (int t = 0; t < S; ++t) {
 #pragma unroll
-            for (int t = 0; t <= L; ++t)
-                tc_mma_lo(tmem + 2 * BN, a0 + t * (BM * 4) + 2 * h, b0 + (L - t) * (BN * 4) + 2 * h, hi, idesc,
-                          (L == 2 && t == 0) ? k0 : 1u);
+            for (int u = 0; u < S - t; ++u) {
+                const int L = t + u;
+                const uint32_t d = tmem + (L < 2 ? L : 2) * BN;
+                const uint32_t a = a0 + t * (BM * 4) + 2 * h, b = b0 + u * (BN * 4) + 2 * h;
+                // the first product into each accumulator: (0, 0), (0, 1), (0, 2)
+                const uint32_t acc = t == 0 && u <= 2 ? k0 : 1u;
+                if (S - t == 1) tc_mma_lo<0>(d, a, b, hi, idesc, acc);
+                else if (u == 0) tc_mma_lo<1>(d, a, b, hi, idesc, acc);
+                else if (u < S - t - 1) tc_mma_lo<2>(d, a, b, hi, idesc, acc);
+                else tc_mma_lo<3>(d, a, b, hi, idesc, acc);
+            }
+        }
     }
 }
 
