@@ -788,33 +788,25 @@ __device__ __forceinline__ bool elect_one() {
     asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
     return p != 0;
 }
-// tc_mma on descriptors given by their low words (address, leading offset).
-// USE: what becomes of the A operand in the collector buffer -- 0 as it
-// comes, 1 kept for the next MMAs, 2 taken from there and kept, 3 taken from
-// there for the last time.
-template <int USE>
+// tc_mma on descriptors given by their low words (address, leading offset)
 __device__ __forceinline__ void tc_mma_lo(uint32_t d_tmem, uint32_t alo, uint32_t blo, uint32_t hi, uint32_t idesc,
                                           uint32_t accumulate) {
-#define CTM_MMA_LO(COLLECTOR)                                                                        \
-    asm volatile(                                                                                    \
-        "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\t"                                                \
-        "mov.b64 da, {%1, %3};\n\tmov.b64 db, {%2, %3};\n\t"                                         \
-        "setp.ne.b32 p, %5, 0;\n\t"                                                                  \
-        "tcgen05.mma.cta_group::1.kind::f16" COLLECTOR " [%0], da, db, %4, p;\n\t}" ::"r"(d_tmem),   \
-        "r"(alo), "r"(blo), "r"(hi), "r"(idesc), "r"(accumulate)                                     \
-        : "memory")
-    if (USE == 0) CTM_MMA_LO("");
-    else if (USE == 1) CTM_MMA_LO(".collector::a::fill");
-    else if (USE == 2) CTM_MMA_LO(".collector::a::use");
-    else CTM_MMA_LO(".collector::a::lastuse");
-#undef CTM_MMA_LO
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\t"
+        "mov.b64 da, {%1, %3};\n\tmov.b64 db, {%2, %3};\n\t"
+        "setp.ne.b32 p, %5, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, p;\n\t}" ::"r"(d_tmem),
+        "r"(alo), "r"(blo), "r"(hi), "r"(idesc), "r"(accumulate)
+        : "memory");
 }
 // All slice products of one 32-wide k-block, S slices: level 0 and level 1 into
 // their accumulators, the rest into the third; keep = 0 restarts the three.
 // Straight-line code on constant offsets from the two tile addresses: issued
 // from loops over runtime slice indices an MMA took 137 cycles whatever its
-// width, so ~100 at N = 144 and 75 at N = 64.  A slice by A slice, so that the
-// 128-row operand is read once for its products instead of once for each.
+// width, so ~100 at N = 144 and 75 at N = 64.  Level by level: the FP32
+// rounding of the third accumulator follows the order.  (A slice by A slice with
+// the operand kept in the collector buffer was 4-10% faster, and its rounding
+// moved observables of small emulated runs by up to 4e-10.)
 template <int S, int BN>
 __device__ __forceinline__ void issue_levels(uint32_t tmem, uint32_t sa, uint32_t sb, uint32_t idesc, uint32_t keep) {
     constexpr uint64_t top = (uint64_t)(512 >> 4) << 32 | (uint64_t)1 << 46 | (uint64_t)4 << 61;  // as sw64_desc
@@ -824,20 +816,14 @@ __device__ __forceinline__ void issue_levels(uint32_t tmem, uint32_t sa, uint32_
     for (int h = 0; h < 2; ++h) {  // two K=16 halves, 32 bytes apart in the 64-byte row
         const uint32_t k0 = h ? 1u : keep;
 #pragma unroll
-        for (int t = 0; t < S; ++t) {
+        for (int L = 0; L < S; ++L)
 #pragma unroll
-            for (int u = 0; u < S - t; ++u) {
-                const int L = t + u;
+            for (int t = 0; t <= L; ++t) {
+                const int u = L - t;
                 const uint32_t d = tmem + (L < 2 ? L : 2) * BN;
                 const uint32_t a = a0 + t * (BM * 4) + 2 * h, b = b0 + u * (BN * 4) + 2 * h;
-                // the first product into each accumulator: (0, 0), (0, 1), (0, 2)
-                const uint32_t acc = t == 0 && u <= 2 ? k0 : 1u;
-                if (S - t == 1) tc_mma_lo<0>(d, a, b, hi, idesc, acc);
-                else if (u == 0) tc_mma_lo<1>(d, a, b, hi, idesc, acc);
-                else if (u < S - t - 1) tc_mma_lo<2>(d, a, b, hi, idesc, acc);
-                else tc_mma_lo<3>(d, a, b, hi, idesc, acc);
+                tc_mma_lo(d, a, b, hi, idesc, t == 0 && u <= 2 ? k0 : 1u);
             }
-        }
     }
 }
 
@@ -1487,17 +1473,19 @@ Plan plan_of(int M, int N, int K, int s, int mode = 0) {
     p.n_tiles = (N + p.bn - 1) / p.bn;
     const int nchunks = (p.nkb + oz::CHUNK_KB - 1) / oz::CHUNK_KB;
     const int tiles = p.m_tiles * p.n_tiles;
-    // Split K when the tiles leave SMs idle (at any 32 of K: the sums are exact
-    // int64): the split whose fullest SM has the least work, 2 s(s+1)/2 MMAs per
-    // k-block, a drain per chunk, and the partials' pass.  64 tiles x 256
-    // k-blocks in 3 splits put 176 k-blocks on some SMs, in 2 splits 128 on all.
+    // Split K when the tiles leave SMs idle, at whole chunks (the FP32 levels are
+    // summed per chunk: splits inside one changed their rounding, and observables
+    // of small emulated runs by 1e-9): the split whose fullest SM has the least
+    // work, 2 s(s+1)/2 MMAs per k-block, a drain per chunk, and the partials'
+    // pass.  64 tiles x 32 chunks in 3 splits put 22 chunks on some SMs, in 2
+    // splits 16 on all.
     int ks = 1;
     if (mode == 0 && tiles < 120 && nchunks >= 2) {
         const double kb = (double)s * (s + 1) * mma_cycles(p.bn);
         double best = -1.0;
-        for (int k = 2; k <= p.nkb && k <= 256; ++k) {
-            const int per = (p.nkb + k - 1) / k;
-            if ((p.nkb + per - 1) / per != k) continue;
+        for (int k = 2; k <= nchunks; ++k) {
+            const int per = (nchunks + k - 1) / k * oz::CHUNK_KB;
+            if ((nchunks * oz::CHUNK_KB + per - 1) / per != k) continue;
             const double cta = per * kb + 2500.0 * ((per + oz::CHUNK_KB - 1) / oz::CHUNK_KB) + 5000.0;
             const double cost = ((tiles * k + 151) / 152) * cta + 8.0 * k * p.m_tiles * oz::BM * p.n_tiles * p.bn / 1500.0;
             if (best < 0.0 || cost < best) {
@@ -1509,7 +1497,7 @@ Plan plan_of(int M, int N, int K, int s, int mode = 0) {
     // int64 sums of a split stay below 2^59 for K <= 16384
     const int max_kb_per_split = 16384 / oz::BK;
     if (mode == 0) ks = std::max(ks, (p.nkb + max_kb_per_split - 1) / max_kb_per_split);
-    p.kb_per_split = mode == 0 ? (p.nkb + ks - 1) / ks : p.nkb;
+    p.kb_per_split = mode == 0 ? (nchunks + ks - 1) / ks * oz::CHUNK_KB : p.nkb;
     p.ksplit = (p.nkb + p.kb_per_split - 1) / p.kb_per_split;
     p.a_bytes = (uint32_t)(s * oz::BM * oz::BK * 2);
     p.stage_bytes = p.a_bytes + (uint32_t)(s * p.bn * oz::BK * 2);
