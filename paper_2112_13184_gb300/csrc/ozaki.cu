@@ -161,9 +161,32 @@ __device__ __forceinline__ double i64_ldexp(long long Z, int E) {
 // 2^9 per chunk, is split by two magic additions of 1.5 2^23 into 6 and 22
 // fractional bits: no conversion of it (an FP32 -> int64 conversion issues on
 // the FP64 pipe, 64 cycles a warp; FP32 -> int32 on the 16-lane one).
-__device__ __forceinline__ long long fixed_add(long long Z, float a0, float a1, float F) {
+// fixed_add_w takes the integer weights as kernel arguments: as literals the
+// compiler turns the 32 x 32 + 64 multiply-adds of the FMA pipe into shifts and
+// adds on the half-rate integer pipe, which bounds the short products'
+// epilogue (262144 x 192 x 64: 171 -> 159 us).  The long products' one is short
+// of registers instead and keeps the literals (8192 x 128 x 8192: 261 us, 290
+// with arguments).
+struct Weights {
+    int w20, w22, w28, one;
+};
+__device__ __forceinline__ long long mad_wide(int a, int b, long long c) {
+    long long d;
+    asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(d) : "r"(a), "r"(b), "l"(c));
+    return d;
+}
+__device__ __forceinline__ long long fixed_add_w(const Weights& w, long long Z, float a0, float a1, float F) {
     const float h = fmaf(F, 64.0f, 12582912.0f);
     const float r = fmaf(F, 64.0f, 12582912.0f - h);  // F 2^6 minus its rounding, exact
+    const float h2 = fmaf(r, 4194304.0f, 12582912.0f);
+    Z = mad_wide(__float_as_int(h2) - 0x4B400000, w.one, Z);
+    Z = mad_wide(__float_as_int(h) - 0x4B400000, w.w22, Z);
+    Z = mad_wide(__float2int_rn(a1 * 256.0f), w.w20, Z);
+    return mad_wide(__float2int_rn(a0), w.w28, Z);
+}
+__device__ __forceinline__ long long fixed_add(long long Z, float a0, float a1, float F) {
+    const float h = fmaf(F, 64.0f, 12582912.0f);
+    const float r = fmaf(F, 64.0f, 12582912.0f - h);
     const float h2 = fmaf(r, 4194304.0f, 12582912.0f);
     const int i1 = __float_as_int(h) - 0x4B400000, i2 = __float_as_int(h2) - 0x4B400000;
     Z += i2;
@@ -176,18 +199,20 @@ __device__ __forceinline__ long long fixed_add(long long Z, float a0, float a1, 
 // the FP64 range from any finite partner
 constexpr int BAD_EXP = 100000;
 __device__ __forceinline__ int safe_exp(int e) { return e > 1024 ? BAD_EXP : e; }
-// Z 2^E where |Z| < 2^53 (exact: a left shift only) and the result is normal
-// or zero; else `bad` is set and the value is meaningless.  No branch: a
-// branch per entry kept the entries of a block from overlapping.
+// Z 2^E where |Z| < 2^53 (exact: a left shift only; SHORT: known to hold) and
+// the result is normal or zero; else `bad` is set and the value is
+// meaningless.  No branch: a branch per entry kept the entries of a block from
+// overlapping.
+template <bool SHORT>
 __device__ __forceinline__ double z_scaled_fast(long long Z, int E, bool& bad) {
     const long long sg = Z >> 63;
     const unsigned long long m = (unsigned long long)((Z ^ sg) - sg);
     const unsigned mh = (unsigned)(m >> 32), ml = (unsigned)m;
     const int c = mh ? __clz((int)mh) : 32 + __clz((int)ml);
-    const int be = c == 64 ? 1 : E + 1086 - c;  // biased exponent of m 2^E; 1 makes a zero come out as zero
-    bad = bad || c < 11 || (unsigned)(be - 1) >= 2046u || E > BAD_EXP / 2;
+    const unsigned be = (unsigned)(E + 1085 - c);  // exponent field of m 2^E minus 1: the implicit bit adds 1
+    bad = bad || be >= 2046u || (!SHORT && c < 11);
     const unsigned long long mant = m << ((c - 11) & 63);  // implicit bit at 52
-    const unsigned hi = (unsigned)(mant >> 32) + ((unsigned)(be - 1) << 20) + ((unsigned)sg & 0x80000000u);
+    const unsigned hi = (unsigned)(mant >> 32) + (m ? be << 20 : 0u) + ((unsigned)sg & 0x80000000u);
     return __hiloint2double((int)hi, (int)(unsigned)mant);
 }
 // larger |Z| (sums of several chunks), results outside the normal range,
@@ -198,7 +223,7 @@ __device__ __noinline__ double z_scaled_slow(long long Z, int E) {
 }
 __device__ __forceinline__ double z_scaled(long long Z, int E) {
     bool bad = false;
-    const double v = z_scaled_fast(Z, E, bad);
+    const double v = z_scaled_fast<false>(Z, E, bad);
     return bad ? z_scaled_slow(Z, E) : v;
 }
 
@@ -843,6 +868,7 @@ struct GemmArgs {
     double alpha, beta;
     double* C;
     View out_r, out_c;    // C offset of (m, n) = view(out_r, m) + view(out_c, n)
+    Weights w;            // of the int64 sums' parts
     int plain;            // alpha = 1 and beta = 0
     int vec;              // 4 or 2: aligned groups of so many columns are contiguous; else 1
     long long* PZ;        // split-K partials [z][Mpad][Npad]
@@ -855,6 +881,7 @@ struct GemmArgs {
 // Eight consecutive output columns from n8 of the lane's row m: built from
 // their int64 sums and stored (crow: the row's output address, ea = row
 // exponent - 44; every lane of the warp calls).
+template <bool SHORT>
 __device__ __forceinline__ void emit8(const GemmArgs& g, const long long* Z, int ea, int m, int n8, double* crow,
                                       int lane) {
     // the columns are the same for every lane: lane j works out column j's
@@ -865,7 +892,7 @@ __device__ __forceinline__ void emit8(const GemmArgs& g, const long long* Z, int
     double v[8];
     bool bad = false;
 #pragma unroll
-    for (int j = 0; j < 8; ++j) v[j] = z_scaled_fast(Z[j], ea + __shfl_sync(0xffffffffu, eb_l, j), bad);
+    for (int j = 0; j < 8; ++j) v[j] = z_scaled_fast<SHORT>(Z[j], ea + __shfl_sync(0xffffffffu, eb_l, j), bad);
     if (__any_sync(0xffffffffu, bad)) {
 #pragma unroll
         for (int j = 0; j < 8; ++j) v[j] = z_scaled(Z[j], ea + __shfl_sync(0xffffffffu, eb_l, j));
@@ -1170,7 +1197,7 @@ __global__ void __launch_bounds__(THREADS, 1)
 #pragma unroll
                 for (int jb = 0; jb < NC; ++jb) {
                     const int b = grp + 3 * jb;
-                    if (b < NB8) emit8(g, Z[jb], ea, m, n0 + b * 8, crow, lane);
+                    if (b < NB8) emit8<false>(g, Z[jb], ea, m, n0 + b * 8, crow, lane);
                 }
             } else {
 #pragma unroll
@@ -1343,9 +1370,9 @@ __global__ void __launch_bounds__(SHORT_THREADS, 1)
                 long long Z[8];
 #pragma unroll
                 for (int j = 0; j < 8; ++j)
-                    Z[j] = fixed_add(0, __uint_as_float(r0[j]), __uint_as_float(r1[j]),
+                    Z[j] = fixed_add_w(g.w, 0, __uint_as_float(r0[j]), __uint_as_float(r1[j]),
                                      g.s > 2 ? __uint_as_float(r2[j]) : 0.0f);
-                emit8(g, Z, ea, m, n0 + b * 8, crow, lane);
+                emit8<true>(g, Z, ea, m, n0 + b * 8, crow, lane);
             }
             if (grp >= NB8) {  // fewer blocks than warps: this one read nothing
                 __syncwarp();
@@ -1747,6 +1774,7 @@ cudaError_t oz_gemm_view(int M, int N, int K, int s, const void* Asplit, const v
     // lane holds a row, and 8-byte stores to 32 rows left every sector written
     // in four parts (262144 x 192 x 64, row-major: 415 us).  Groups of `vec`
     // columns must be contiguous and aligned for every row.
+    g.w = oz::Weights{1 << 20, 1 << 22, 1 << 28, 1};
     g.plain = alpha == 1.0 && beta == 0.0;
     g.vec = 1;
     if (g.plain)
