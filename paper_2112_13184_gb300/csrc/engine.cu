@@ -101,14 +101,17 @@ struct ctm_ctx {
     double *Lh = nullptr, *Rh = nullptr, *rho = nullptr, *spec = nullptr, *corners = nullptr;
     double* splitk = nullptr;  // split-K partial sums
     size_t splitk_n = 0;
-    // Second branch of a column step (small handles): the two cuts' range
-    // finders, and their projectors, run side by side on two streams.  The
-    // scratch of the second; BranchScope exchanges it with the fields above
-    // and below while that branch's calls are issued.
+    // Second branch of a column step (small handles): the enlarged corners, the
+    // two cuts' range finders and projectors, and the two absorptions run side
+    // by side on two streams.  The scratch of the second; BranchScope exchanges
+    // it with the handle's own while that branch's calls are issued.
     struct Branch {
         cudaStream_t stream = nullptr;
         double *Om = nullptr, *Yb = nullptr, *Zb = nullptr, *Qm2 = nullptr, *Rb = nullptr, *Uc = nullptr, *Vc = nullptr;
         double *t1 = nullptr, *t2 = nullptr, *inv = nullptr, *splitk = nullptr;
+        double *X1 = nullptr, *S1 = nullptr, *S2 = nullptr, *newC1 = nullptr, *newC4 = nullptr, *newT4 = nullptr;
+        double* tmpT = nullptr;
+        unsigned long long* maxbits = nullptr;
         size_t splitk_n = 0, ozA_n = 0, ozB_n = 0, ozW_n = 0;
         void *ozA = nullptr, *ozB = nullptr, *ozW = nullptr, *qr_ws = nullptr;
     } br;
@@ -250,15 +253,18 @@ bool forks(int N, int k, const ctm_options& o) { return o.batch_cuts && ctm::qr_
 struct BranchSizes {
     size_t Nk, kk, tk, splitk, ozA = 0, ozB = 0, ozW = 0;
 };
-BranchSizes branch_sizes(int N, int chi, int k, const ctm_options& o) {
+BranchSizes branch_sizes(int d, int D, int chi, int k, const ctm_options& o) {
     BranchSizes z;
+    const int N = chi * D * D, D2 = D * D, M3 = chi * chi * D2;
     z.Nk = (size_t)N * k;
     z.kk = (size_t)k * k;
     z.tk = (size_t)N * std::max(k, chi);
     z.splitk = 32 * z.tk;
     const int mode = tc_mode_of(o.precision), s = tc_slices_of(o);
     if (mode >= 0) {
-        const int shapes[4][3] = {{N, k, N}, {N, chi, N}, {N, chi, k}, {N, k, k}};
+        // the products of a sweep (gemm_shapes without the density matrices')
+        const int shapes[][3] = {{chi, N, chi}, {N, N, chi}, {M3, d * D2, D2}, {M3, D2, d * D2}, {N, k, N}, {N, chi, N},
+                                 {N, chi, k},   {N, k, k},   {chi, chi, N},    {chi, N, N},      {N, chi, chi}};
         for (const auto& h : shapes) {
             z.ozA = std::max(z.ozA, tc_split_bytes(h[0], h[2], mode, s));
             z.ozB = std::max(z.ozB, tc_split_bytes(h[1], h[2], mode, s));
@@ -730,6 +736,14 @@ struct BranchScope {
         std::swap(h->t1, b.t1);
         std::swap(h->t2, b.t2);
         std::swap(h->inv, b.inv);
+        std::swap(h->X1, b.X1);
+        std::swap(h->S1, b.S1);
+        std::swap(h->S2, b.S2);
+        std::swap(h->newC1, b.newC1);
+        std::swap(h->newC4, b.newC4);
+        std::swap(h->newT4, b.newT4);
+        std::swap(h->tmpT, b.tmpT);
+        std::swap(h->maxbits, b.maxbits);
         std::swap(h->splitk, b.splitk);
         std::swap(h->splitk_n, b.splitk_n);
         std::swap(h->ozA, b.ozA);
@@ -809,12 +823,16 @@ ctm_status resident_corners(ctm_ctx* h, const int* ids, Keep keep) {
         }
         h->E[r] = h->Eb[at[r]];
     }
-    for (int r = 0; r < 8; ++r)
-        if (fresh[r]) {
-            h->eb_corner[at[r]] = ids[r];
-            CKS(enlarged_corner(h, ids[r] / 4, ids[r] & 3, h->E[r]));
-        }
-    return CTM_OK;
+    // the new ones, every other one on the second branch
+    return both_cuts(h, [&](int branch) -> ctm_status {
+        int n = 0;
+        for (int r = 0; r < 8; ++r)
+            if (fresh[r] && n++ % 2 == branch) {
+                h->eb_corner[at[r]] = ids[r];
+                CKS(enlarged_corner(h, ids[r] / 4, ids[r] & 3, h->E[r]));
+            }
+        return CTM_OK;
+    });
 }
 
 ctm_status normalise_into(ctm_ctx* h, const double* src, double* dst, size_t n, int slot) {
@@ -856,12 +874,14 @@ ctm_status left_move(ctm_ctx* h, int m, int x) {
             CKS(projectors(h, y, cut_of(y)));
         }
     }
-    ProfTag tg(h, "absorb");
     // the upper-left corner of the first cut is not needed any more: its buffer
-    // is the absorption's scratch
+    // is the absorptions' scratch, that of the second cut's (which the next
+    // move may still take) only where the two run side by side
+    double* const scratch[2] = {h->E[0], h->fork ? h->E[4] : h->E[0]};
     for (int b = 0; b < h->n_eb; ++b)
-        if (h->Eb[b] == h->E[0]) h->eb_corner[b] = -1;
-    for (int y = 0; y < 2; ++y) {
+        if (h->Eb[b] == scratch[0] || h->Eb[b] == scratch[1]) h->eb_corner[b] = -1;
+    return both_cuts(h, [&](int y) -> ctm_status {
+        ProfTag tg(h, "absorb");
         const int i = FM.site(m, x, y), j = FM.site(m, x + 1, y);
         const int ym = (y + 1) % 2;  // cut between rows y-1 and y
         double** e = h->env[i];
@@ -869,8 +889,8 @@ ctm_status left_move(ctm_ctx* h, int m, int x) {
         CKS(gemm(h, false, false, chi, N, chi, e[Cw(m)], chi, e[Tw(m)], N, h->X1, N));
         CKS(gemm(h, true, false, chi, chi, N, h->Pup[y], chi, h->X1, chi, h->newC1, chi));
         // T4' = P_up(y-1)^T core(P_dn(y)^T, T4, A)   -> [c1, c2, r, r'] -> [c1, r, r', c2]
-        CKS(corner_core(h, h->PdnT[y], e[Tw(m + 3)], h->A[i][m & 3], h->Alu[i][m & 3], h->E[0], false));
-        CKS(gemm(h, true, false, chi, N, N, h->Pup[ym], chi, h->E[0], N, h->tmpT, N));
+        CKS(corner_core(h, h->PdnT[y], e[Tw(m + 3)], h->A[i][m & 3], h->Alu[i][m & 3], scratch[y], false));
+        CKS(gemm(h, true, false, chi, N, N, h->Pup[ym], chi, scratch[y], N, h->tmpT, N));
         CKS(perm(h, h->tmpT, h->newT4, {chi, chi, D, D}, {0, 2, 3, 1}));
         // C4' = (C4 T3)^T P_dn(y-1)^T :  Z[z,d,d',g] = T3[(z,d,d'),h] C4[h,g] -> [z,g,d,d']
         CKS(gemm(h, false, false, N, chi, chi, e[Tw(m + 2)], chi, e[Cw(m + 3)], chi, h->t1, chi));
@@ -882,8 +902,8 @@ ctm_status left_move(ctm_ctx* h, int m, int x) {
         CKS(normalise_into(h, h->newC4, ej[Cw(m + 3)], (size_t)chi * chi, 2));
         for (int b = 0; b < h->n_eb; ++b)
             if (h->eb_corner[b] == corner_id(j, m) || h->eb_corner[b] == corner_id(j, m + 3)) h->eb_corner[b] = -1;
-    }
-    return CTM_OK;
+        return CTM_OK;
+    });
 }
 
 ctm_status one_sweep_eager(ctm_ctx* h) {
@@ -1656,9 +1676,9 @@ ctm_status create(int Lx, int Ly, int d, int D, const ctm_options* o, void* stre
     h->splitk_n = (size_t)1 << 24;
     A_(&h->splitk, h->splitk_n);
     if (st == CTM_OK && forks(h->N, h->k, *o)) {
-        // the second branch's scratch is the tail of the split-K partials' buffer,
+        // the second branch's scratch is the head of the split-K partials' buffer,
         // which no product of a handle this small fills
-        const BranchSizes b = branch_sizes(h->N, h->chi, h->k, *o);
+        const BranchSizes b = branch_sizes(d, D, h->chi, h->k, *o);
         auto& r = h->br;
         size_t used = 0;
         auto take = [&](size_t bytes) {
@@ -1671,13 +1691,16 @@ ctm_status create(int Lx, int Ly, int d, int D, const ctm_options* o, void* stre
         r.Om = dbl(b.Nk), r.Yb = dbl(b.Nk), r.Zb = dbl(b.Nk), r.Qm2 = dbl(b.Nk), r.Vc = dbl(b.Nk), r.Rb = dbl(b.kk);
         r.Uc = dbl(b.tk), r.t1 = dbl(b.tk), r.t2 = dbl(b.tk), r.inv = dbl(h->k), r.splitk = dbl(b.splitk);
         r.splitk_n = b.splitk;
+        r.X1 = dbl(z.T), r.newT4 = dbl(z.T), r.tmpT = dbl(z.T), r.newC1 = dbl(z.C), r.newC4 = dbl(z.C);
+        r.S1 = h->S1 + d * z.NN;  // a sweep's corners use d N^2 of the d^2 N^2 there
+        r.S2 = dbl(d * z.NN);
         r.qr_ws = take(qr_ws_bytes(h->N, h->k));
         if (tc_mode_of(o->precision) >= 0) {
             r.ozA = take(r.ozA_n = b.ozA);
             r.ozB = take(r.ozB_n = b.ozB);
             r.ozW = take(r.ozW_n = b.ozW);
         }
-        if (used <= h->splitk_n * sizeof(double) / 2) {
+        if (d >= 2 && used <= h->splitk_n * sizeof(double) / 4 * 3) {
             h->splitk = whole + used / sizeof(double);
             h->splitk_n -= used / sizeof(double);
             if (cudaStreamCreateWithFlags(&r.stream, cudaStreamNonBlocking) != cudaSuccess ||
@@ -1695,6 +1718,7 @@ ctm_status create(int Lx, int Ly, int d, int D, const ctm_options* o, void* stre
     if (st == CTM_OK) st = alloc(h, &h->svd_ws, svd_ws_bytes(h->k));
     if (st == CTM_OK) st = alloc(h, &h->sval_ws, svals_ws_bytes(h->chi, 16));
     if (st == CTM_OK) st = alloc(h, (void**)&h->maxbits, 64 * sizeof(unsigned long long));
+    h->br.maxbits = h->maxbits + 32;
     if (st == CTM_OK) st = alloc(h, (void**)&h->flag, 64);
     if (st == CTM_OK) st = allocd(h, &h->dotws, ctm::dot_ws_doubles());
     if (st == CTM_OK) st = allocd(h, &h->scal, 8);
