@@ -22,6 +22,7 @@
 // 2^-36 max|row| max|col| K; so 5 slices reach ~1e-11 relative per unit K
 // and a 6th adds nothing.  Split-BF16 accumulated in FP32 over all of K
 // cannot go below ~2^-24.
+#include <cooperative_groups.h>
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -33,6 +34,8 @@
 #include <mutex>
 
 #include "internal.h"
+
+namespace cg = cooperative_groups;
 
 namespace ctm {
 namespace oz {
@@ -630,14 +633,14 @@ __global__ void __launch_bounds__(64) k_split_cols(const double* __restrict__ X,
     }
 }
 
-// The same for K up to COLS_ONE_MAX in one launch, one CTA per 32 rows: its
-// warps (one per 32 k, at most 16) first agree on the row maxima, then
-// slice; the last 32 k a warp read stay in registers, so that K <= 512 is
-// read once.  The three launches of the long form (clear, maxima, slices)
-// cost a small operand more than its bytes: with 32-warp grids the transposed
-// 512 x 512 corner of D=4, chi=32 took ~48 us, and the scan point there went
-// from 107 to 60 ms.  Beyond 1536 the two re-reads per warp cost more than
-// the launches, and short operands leave SMs idle.
+// The same in one launch: a cluster of CTAs takes 32 rows, each of its warps
+// 32 k at a time.  The warps agree on the row maxima (a maximum for each CTA,
+// pushed to every other through distributed shared memory) and slice; the last
+// 32 k a warp read stay in registers, so that K up to 512 times the cluster's
+// CTAs is read once.  What bounds small operands is the integer work of
+// slicing on few SMs, the launches of the long form (clear, maxima, slices)
+// and its second read; large ones HBM, and there one CTA of 16 warps per SM,
+// with its loads and its slicing one after the other, loses to the long form.
 constexpr int COLS_ONE_MAX = 1536;
 constexpr int COLS_ONE_WARPS = 16;
 template <bool PLAIN>
@@ -646,16 +649,20 @@ __global__ void __launch_bounds__(32 * COLS_ONE_WARPS) k_split_cols_one(const do
                                                                        __nv_bfloat16* __restrict__ out,
                                                                        int* __restrict__ ex) {
     __shared__ uint4 tile[COLS_ONE_WARPS][32][5];
-    __shared__ unsigned long long red[COLS_ONE_WARPS][32];
+    __shared__ unsigned long long red[COLS_ONE_WARPS][32], all[16][32];  // of the warps; of the cluster's CTAs
+    cg::cluster_group cl = cg::this_cluster();
     const int w = threadIdx.x >> 5, nw = blockDim.x >> 5, lane = threadIdx.x & 31;
-    const int r0 = blockIdx.x * 32, r = r0 + lane;
+    const int nc = (int)cl.num_blocks(), c = (int)cl.block_rank();
+    if (nc > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+    const int r0 = (int)(blockIdx.x / nc) * 32, r = r0 + lane;
     const bool live = r < R;
     const unsigned long long* xr =
         reinterpret_cast<const unsigned long long*>(X) + (live ? view_offset32(rv, (unsigned)r) : 0);
+    const int step = nc * nw * 32;
     unsigned long long v[32];
     unsigned long long mb = 0;
-    int k0 = w * 32, last = -1;
-    for (; k0 < K8; k0 += nw * 32) {
+    int k0 = (c * nw + w) * 32, last = -1;
+    for (; k0 < K8; k0 += step) {
         load32<PLAIN>(xr, live, k0, K, kv, v);
 #pragma unroll
         for (int u = 0; u < 32; ++u) mb = umax64(mb, v[u] & 0x7fffffffffffffffull);
@@ -663,14 +670,25 @@ __global__ void __launch_bounds__(32 * COLS_ONE_WARPS) k_split_cols_one(const do
     }
     red[w][lane] = mb;
     __syncthreads();
+    if (nc > 1) {
+        // every CTA of the cluster runs before its shared memory is written to
+        asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
+        if (w < nc) {
+            mb = 0;
+            for (int i = 0; i < nw; ++i) mb = umax64(mb, red[i][lane]);
+            for (int i = w; i < nc; i += nw) cl.map_shared_rank(&all[0][0], i)[c * 32 + lane] = mb;
+        }
+        cl.sync();
+    }
     mb = 0;
-    for (int i = 0; i < nw; ++i) mb = umax64(mb, red[i][lane]);
+    const int n = nc > 1 ? nc : nw;
+    for (int i = 0; i < n; ++i) mb = umax64(mb, nc > 1 ? all[i][lane] : red[i][lane]);
     const int e = row_exponent_bits(mb);
-    if (live && w == 0) ex[r] = e;
+    if (live && w == 0 && c == 0) ex[r] = e;
     const size_t plane = (size_t)R * K8;
     const int base = 1075 - 8 * s + e;
     const unsigned long long bias = digit_bias(s);
-    for (k0 = last; k0 >= 0; k0 -= nw * 32) {
+    for (k0 = last; k0 >= 0; k0 -= step) {
         if (k0 != last) load32<PLAIN>(xr, live, k0, K, kv, v);
 #pragma unroll
         for (int u = 0; u < 32; ++u) v[u] = digit_bytes(v[u], base, bias);
@@ -1595,11 +1613,64 @@ inline const int* split_tf32_exponents(const void* buf, int R, int K4) {
 
 // K range of one warp in the lane = row kernels: 256, halved down to 32 until
 // the operand gives every SM sixteen warps
+// Whether the device runs clusters of 16 CTAs of the one-launch slicer (a
+// property of the device: asked once for each).
+static bool cols_cluster_of_16() {
+    static std::mutex mu;
+    static unsigned long long asked = 0, yes = 0;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return false;
+    std::lock_guard<std::mutex> lock(mu);
+    if (asked >> dev & 1ull) return yes >> dev & 1ull;
+    bool ok = true;
+    for (auto k : {oz::k_split_cols_one<true>, oz::k_split_cols_one<false>}) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(16, 1, 1);
+        cfg.blockDim = dim3(32 * oz::COLS_ONE_WARPS, 1, 1);
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = 16;
+        at[0].val.clusterDim.y = 1;
+        at[0].val.clusterDim.z = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        int n = 0;
+        ok = ok && cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+             cudaOccupancyMaxActiveClusters(&n, k, &cfg) == cudaSuccess && n > 0;
+    }
+    if (!ok) cudaGetLastError();
+    asked |= 1ull << dev;
+    yes |= (unsigned long long)ok << dev;
+    return ok;
+}
+
 static int cols_krange(int R, int K) {
     const long long rg = (R + 31) / 32;
     int range = 256;
     while (range > 32 && rg * ((K + range - 1) / range) < 152 * 16) range /= 2;
     return range;
+}
+
+// CTAs of the cluster that slices 32 rows in one launch, 0 where the operand
+// goes the long way (maxima, then slices).  Whole products of 5 slices with
+// such an A, in us, without clusters (K <= 1536: one CTA; above: the long way)
+// and with them, M x N x K:
+//   48x48x1200 57.0, 40.6   1200x48x1200 61.1, 54.9   1024x40x1024 52.9, 42.8
+//   144x144x8192 76.4, 67.2   2048x64x2048 72.3, 63.1   20000x64x2048 430, 407
+//   8192x144x1536 153, 168   30000x16x1200 302, 346   8192x144x5000 530, 557
+// so clusters of 16 and those of short rows (K <= 1536) are for operands of one
+// wave or two, clusters of up to 8 for K in between whatever R.
+static int cols_cluster(int R, int K8) {
+    const long long rg = (R + 31) / 32;
+    const int warps = (K8 + 31) / 32;
+    const bool small = rg * warps <= 152 * 2 * oz::COLS_ONE_WARPS;
+    if (!small && K8 <= oz::COLS_ONE_MAX) return 1;
+    int nc = 1;
+    while (nc < 16 && nc * oz::COLS_ONE_WARPS < warps) nc *= 2;
+    if (nc * oz::COLS_ONE_WARPS < warps || rg * nc > 0x7fffffffll) return 0;
+    if (nc == 16) return small && cols_cluster_of_16() ? 16 : 0;
+    while (nc < 8 && rg * nc < 152 && nc * 2 < warps) nc *= 2;
+    return nc;
 }
 
 cudaError_t oz_split_tf32(const double* X, int R, int K, const OzView& rvh, const OzView& kvh, void* buf,
@@ -1695,12 +1766,22 @@ cudaError_t oz_split_view(const double* X, int R, int K, const OzView& rvh, cons
         oz::k_rowmax_rows<<<(unsigned)b1, 256, 0, st>>>(X, R, K, rv, kv, kr, mb);
         ++g_launches;
         oz::k_split_rows_long<<<(unsigned)b2, 256, 0, st>>>(X, R, K, K8, rv, kv, s, mb, sl, ex);
-    } else if (K8 <= oz::COLS_ONE_MAX) {
-        const unsigned rg = (unsigned)((R + 31) / 32);
-        const int nw = std::min(oz::COLS_ONE_WARPS, (K8 + 31) / 32);
+    } else if (const int nc = cols_cluster(R, K8)) {
+        const int warps = std::min(oz::COLS_ONE_WARPS, ((K8 + 31) / 32 + nc - 1) / nc);
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)((R + 31) / 32 * nc), 1, 1);
+        cfg.blockDim = dim3((unsigned)(32 * warps), 1, 1);
+        cfg.stream = st;
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = (unsigned)nc;
+        at[0].val.clusterDim.y = 1;
+        at[0].val.clusterDim.z = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
         ++g_launches;
-        if (kv.n == 1) oz::k_split_cols_one<true><<<rg, 32 * nw, 0, st>>>(X, R, K, K8, rv, kv, s, sl, ex);
-        else oz::k_split_cols_one<false><<<rg, 32 * nw, 0, st>>>(X, R, K, K8, rv, kv, s, sl, ex);
+        return cudaLaunchKernelEx(&cfg, kv.n == 1 ? oz::k_split_cols_one<true> : oz::k_split_cols_one<false>, X, R, K, K8,
+                                  rv, kv, s, sl, ex);
     } else {
         cudaError_t e = cudaMemsetAsync(mb, 0, (size_t)R * 8, st);
         if (e != cudaSuccess) return e;

@@ -76,3 +76,19 @@ def test_slices_of_every_magnitude(ctm, slices):
     # rounding shows (the documented 2^-36)
     tol = 2.0 ** -43 if slices < 6 else 2.0 ** -36
     assert np.all(np.abs(C.cpu().numpy() - want) <= np.ldexp(tol, e)[:, None])
+
+
+@pytest.mark.parametrize("M,N,K", [(33, 2, 1537), (1, 1, 4096), (65, 3, 4097), (31, 1, 8191), (48, 5, 1200), (640, 1, 511),
+                                   (2, 1, 300), (5000, 1, 1536), (40000, 1, 530), (9000, 1, 4090), (1300, 1, 8192)])
+def test_column_slicer_clusters(ctm, M, N, K):
+    """A read along its rows' contiguous direction: clusters of 2 to 16, one CTA and the long form.  The
+    only large entry of a row sits at its last k, so that a CTA without the cluster's maximum goes wrong."""
+    rng = np.random.default_rng(M + K)
+    A = rng.integers(-1, 2, size=(K, M)).astype(np.float64)
+    A[K - 1, :] = 60000.0
+    B = rng.integers(-255, 256, size=(K, N)).astype(np.float64)
+    C = torch.empty((M, N), dtype=torch.float64, device="cuda")
+    ws = torch.zeros(ctm.ctm_gemm_ozaki_workspace_bytes(M, N, K, 2), dtype=torch.uint8, device="cuda")
+    ctm.ctm_gemm_ozaki(1, 0, M, N, K, 1.0, torch.from_numpy(A).cuda(), M, torch.from_numpy(B).cuda(), N, 0.0, C, N, 2, ws)
+    torch.cuda.synchronize()
+    np.testing.assert_array_equal(C.cpu().numpy(), A.T @ B)
