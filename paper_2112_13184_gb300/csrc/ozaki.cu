@@ -337,35 +337,61 @@ __device__ __forceinline__ unsigned slice_of_pair(unsigned long long za, unsigne
     return digit_pair(__byte_perm(a, b, (byte & 3) | ((4 + (byte & 3)) << 8)), t);
 }
 
-// Per-row max|x| of operands whose rows are not contiguous in k: lane = row,
-// a warp takes 32 rows x `krange` k, combined with atomicMax on the bit
-// patterns (non-negative doubles order like integers).
-__global__ void k_rowmax_cols(const double* __restrict__ X, int R, int K, View rv, View kv, int kranges, int krange,
-                              unsigned long long* __restrict__ maxbits) {
+// Per-row maxima of operands whose rows are not contiguous in k, as bit
+// patterns that have the exponent of max|x| and are zero only where it is (all
+// that row_exponent_bits asks for): lane = row, a warp takes 32 rows x
+// `krange` k, combined with atomicMax (non-negative doubles order like
+// integers).  PLAIN: one K stride.  Bound by HBM: three integer instructions an
+// element on its two words and 16 loads in flight per lane.  (8 loads and an
+// odometer step for each: 147 us for the 537 MB of 8192 x 8192, about 85 now;
+// a whole 8192 x 16 x 8192 product 548 -> 484.)
+template <bool PLAIN>
+__global__ void __launch_bounds__(128) k_rowmax_cols(const double* __restrict__ X, int R, int K, View rv, View kv,
+                                                     int kranges, int krange, unsigned long long* __restrict__ maxbits) {
     const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     const int rg = w / kranges, kr = w - rg * kranges;
     const int r = rg * 32 + lane;
     const int k0 = kr * krange;
     if (r >= R || k0 >= K) return;
     const int k1 = min(K, k0 + krange);
-    const double* xr = X + view_offset32(rv, (unsigned)r);
-    Odometer od;
-    od.init(kv, (unsigned)k0);
-    unsigned long long mx = 0;
-    for (int k = k0; k < k1; k += 8) {
-        long long off[8];
+    const int2* xr = reinterpret_cast<const int2*>(X) + view_offset32(rv, (unsigned)r);
+    int hi = 0, lo = 0;
+    int k = k0;
+    auto take = [&](const int2* v) {
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            off[u] = od.off;
-            if (k + u + 1 < k1) od.step(kv);
+        for (int u = 0; u < 16; ++u) {
+            hi = max(hi, v[u].y & 0x7fffffff);
+            lo |= v[u].x;
         }
-        double v[8];
+    };
+    if (PLAIN) {
+        const long long cs = kv.stride[0];
+        xr += k0 * cs;
+        for (; k + 16 <= k1; k += 16, xr += 16 * cs) {
+            int2 v[16];
 #pragma unroll
-        for (int u = 0; u < 8; ++u) v[u] = (k + u < k1) ? xr[off[u]] : 0.0;
+            for (int u = 0; u < 16; ++u) v[u] = __ldg(xr + u * cs);
+            take(v);
+        }
+        for (; k < k1; ++k, xr += cs) {
+            const int2 v = __ldg(xr);
+            hi = max(hi, v.y & 0x7fffffff);
+            lo |= v.x;
+        }
+    } else {
+        Odometer od;
+        od.init(kv, (unsigned)k0);
+        for (; k < k1; k += 16) {
+            int2 v[16];
 #pragma unroll
-        for (int u = 0; u < 8; ++u) mx = umax64(mx, abs_bits(v[u]));
+            for (int u = 0; u < 16; ++u) {
+                v[u] = k + u < k1 ? __ldg(xr + od.off) : make_int2(0, 0);
+                if (k + u + 1 < k1) od.step(kv);
+            }
+            take(v);
+        }
     }
-    atomicMax(maxbits + r, mx);
+    atomicMax(maxbits + r, (unsigned long long)hi << 32 | (lo != 0));
 }
 
 // round(x 2^(nbits - e)) as an integer, |x| <= 2^e (integer operations on the
@@ -604,9 +630,12 @@ __device__ __forceinline__ void load32(const unsigned long long* xr, bool live, 
 
 // Operands read along their rows' contiguous direction (lane = row): one
 // warp per 32 rows x kspan k (kspan a multiple of 32), row maxima from
-// k_rowmax_cols.  PLAIN: one K stride.
+// k_rowmax_cols.  PLAIN: one K stride.  Bound by HBM; warps of 64 k at most
+// and 16 of them on an SM keep the last wave short: 8192 x 16 x 8192 485 -> 477
+// us, 5000 x 16 x 6000 265 -> 245 against 256 k and 12 warps.
+constexpr int COLS_SPAN = 64;
 template <bool PLAIN>
-__global__ void __launch_bounds__(64) k_split_cols(const double* __restrict__ X, int R, int K, int K8, View rv, View kv,
+__global__ void __launch_bounds__(64, 8) k_split_cols(const double* __restrict__ X, int R, int K, int K8, View rv, View kv,
                                                   int s, const unsigned long long* __restrict__ maxbits,
                                                   __nv_bfloat16* __restrict__ out, int* __restrict__ ex, int kspan,
                                                   int kgroups) {
@@ -1673,6 +1702,12 @@ static int cols_cluster(int R, int K8) {
     return nc;
 }
 
+static void launch_rowmax_cols(unsigned blocks, cudaStream_t st, const double* X, int R, int K, const oz::View& rv,
+                               const oz::View& kv, int kranges, int krange, unsigned long long* mb) {
+    if (kv.n == 1) oz::k_rowmax_cols<true><<<blocks, 128, 0, st>>>(X, R, K, rv, kv, kranges, krange, mb);
+    else oz::k_rowmax_cols<false><<<blocks, 128, 0, st>>>(X, R, K, rv, kv, kranges, krange, mb);
+}
+
 cudaError_t oz_split_tf32(const double* X, int R, int K, const OzView& rvh, const OzView& kvh, void* buf,
                           cudaStream_t st) {
     if (R <= 0 || K <= 0 || rvh.n < 1 || rvh.n > 4 || kvh.n < 1 || kvh.n > 4) return cudaErrorInvalidValue;
@@ -1698,7 +1733,7 @@ cudaError_t oz_split_tf32(const double* X, int R, int K, const OzView& rvh, cons
     const unsigned long long threads = (unsigned long long)R * (K4 / 4);
     if ((warps + 3) / 4 > 0x7fffffffull || (threads + 255) / 256 > 0x7fffffffull) return cudaErrorInvalidValue;
     ++g_launches;
-    oz::k_rowmax_cols<<<(unsigned)((warps + 3) / 4), 128, 0, st>>>(X, R, K, rv, kv, (int)kr, krange, mb);
+    launch_rowmax_cols((unsigned)((warps + 3) / 4), st, X, R, K, rv, kv, (int)kr, krange, mb);
     ++g_launches;
     oz::k_split_tf32<<<(unsigned)((threads + 255) / 256), 256, 0, st>>>(X, R, K, K4, rv, kv, mb, sl, ex);
     return cudaGetLastError();
@@ -1789,11 +1824,11 @@ cudaError_t oz_split_view(const double* X, int R, int K, const OzView& rvh, cons
         const int krange = cols_krange(R, K);
         const unsigned kr = (unsigned)((K + krange - 1) / krange);
         const unsigned long long warps = (unsigned long long)rg * kr;
-        const int kspan = cols_krange(R, K8), kgroups = (K8 + kspan - 1) / kspan;
+        const int kspan = std::min(oz::COLS_SPAN, cols_krange(R, K8)), kgroups = (K8 + kspan - 1) / kspan;
         const unsigned long long warps2 = (unsigned long long)rg * kgroups;
         if ((warps + 3) / 4 > 0x7fffffffull || (warps2 + 1) / 2 > 0x7fffffffull) return cudaErrorInvalidValue;
         ++g_launches;
-        oz::k_rowmax_cols<<<(unsigned)((warps + 3) / 4), 128, 0, st>>>(X, R, K, rv, kv, (int)kr, krange, mb);
+        launch_rowmax_cols((unsigned)((warps + 3) / 4), st, X, R, K, rv, kv, (int)kr, krange, mb);
         const unsigned blocks = (unsigned)((warps2 + 1) / 2);
         ++g_launches;
         if (kv.n == 1) oz::k_split_cols<true><<<blocks, 64, 0, st>>>(X, R, K, K8, rv, kv, s, mb, sl, ex, kspan, kgroups);
