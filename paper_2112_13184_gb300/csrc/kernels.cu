@@ -36,6 +36,7 @@ __global__ void __launch_bounds__(256) k_dgemm(int M, int N, int K, double alpha
                                                long long sam, long long sak, const double* __restrict__ B,
                                                long long sbk, long long sbn, double beta, double* __restrict__ C,
                                                int ldc, int kchunk, size_t zstride) {
+    dep_wait(A, B, C);
     constexpr int BM = 32 * TM, BN = 8 * TN;
     constexpr int NA = BM * GK / 256, NB = (BN * GK + 255) / 256;
     __shared__ double As[GK][BM + 1];
@@ -115,6 +116,7 @@ __global__ void __launch_bounds__(256) k_dgemm(int M, int N, int K, double alpha
 }
 __global__ void k_splitk_reduce(const double* __restrict__ P, int splits, int M, int N, double alpha,
                                 double beta, double* __restrict__ C, int ldc) {
+    dep_wait(P, C);
     const size_t total = (size_t)M * N;
     for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < total; t += (size_t)gridDim.x * blockDim.x) {
         double acc = 0.0;
@@ -136,6 +138,7 @@ constexpr int GEMV_ROWS = 16;
 constexpr int GEMV_CTAS = 152 * 4;
 __global__ void __launch_bounds__(256) k_gemv_long(int M, int K, const double* __restrict__ A, int lda,
                                                    const double* __restrict__ x, int incx, double* __restrict__ P) {
+    dep_wait(A, x, P);
     __shared__ double sm[8][GEMV_ROWS];
     double acc[GEMV_ROWS];
 #pragma unroll
@@ -164,6 +167,7 @@ __global__ void __launch_bounds__(256) k_gemv_long(int M, int K, const double* _
 
 __global__ void k_gemv_sum(const double* __restrict__ P, int parts, int M, double alpha, double beta,
                            double* __restrict__ C, int ldc) {
+    dep_wait(P, C);
     const int m = threadIdx.x >> 5, lane = threadIdx.x & 31;
     double t = 0.0;
 #pragma unroll 4
@@ -223,9 +227,8 @@ struct GemmArgs64 {
 };
 template <int TM, int TN>
 void launch(dim3 g, cudaStream_t s, const GemmArgs64& a) {
-    ++g_launches;
-    k_dgemm<TM, TN><<<g, 256, 0, s>>>(a.M, a.N, a.K, a.alpha, a.A, a.sam, a.sak, a.B, a.sbk, a.sbn, a.beta, a.C, a.ldc,
-                                      a.kchunk, a.zs);
+    launch_dep(k_dgemm<TM, TN>, g, 256, 0, s, a.M, a.N, a.K, a.alpha, a.A, a.sam, a.sak, a.B, a.sbk, a.sbn, a.beta, a.C,
+               a.ldc, a.kchunk, a.zs);
 }
 template <int TM>
 void launch_tn(int tn, dim3 g, cudaStream_t s, const GemmArgs64& a) {
@@ -248,10 +251,8 @@ cudaError_t dgemm(bool tA, bool tB, int M, int N, int K, double alpha, const dou
                   size_t ws_doubles) {
     if (M <= 0 || N <= 0) return cudaSuccess;
     if (N == 1 && !tA && M <= GEMV_ROWS && K >= (1 << 16) && ws && ws_doubles >= (size_t)GEMV_CTAS * M) {
-        ++g_launches;
-        k_gemv_long<<<GEMV_CTAS, 256, 0, s>>>(M, K, A, lda, B, tB ? 1 : ldb, ws);
-        ++g_launches;
-        k_gemv_sum<<<1, 32 * M, 0, s>>>(ws, GEMV_CTAS, M, alpha, beta, C, ldc);
+        launch_dep(k_gemv_long, GEMV_CTAS, 256, 0, s, M, K, A, lda, B, tB ? 1 : ldb, ws);
+        launch_dep(k_gemv_sum, 1, 32 * M, 0, s, ws, GEMV_CTAS, M, alpha, beta, C, ldc);
         return cudaGetLastError();
     }
     const GemmPlan p = dgemm_plan(M, N, K, ws ? ws_doubles : 0);
@@ -274,8 +275,7 @@ cudaError_t dgemm(bool tA, bool tB, int M, int N, int K, double alpha, const dou
     if (p.splits > 1) {
         size_t blocks = ((size_t)M * N + 255) / 256;
         if (blocks > 152 * 8) blocks = 152 * 8;
-        ++g_launches;
-        k_splitk_reduce<<<(unsigned)blocks, 256, 0, s>>>(ws, p.splits, M, N, alpha, beta, C, ldc);
+        launch_dep(k_splitk_reduce, (unsigned)blocks, 256, 0, s, ws, p.splits, M, N, alpha, beta, C, ldc);
     }
     return cudaGetLastError();
 }
@@ -301,6 +301,7 @@ struct GatherArgs {
 };
 __global__ void k_permute_gather(const double* __restrict__ src, double* __restrict__ dst, unsigned total,
                                  const GatherArgs p) {
+    dep_wait(src, dst);
     const unsigned o = blockIdx.x * 256 + threadIdx.x;
     if (o >= total) return;
     unsigned rem = o, off = 0;
@@ -366,6 +367,7 @@ k_permute(const double* __restrict__ src, double* __restrict__ dst, const __grid
         sidx[i] = perm_digits(p.src, p.n_in, e, soff[i], pos);
         spos[i] = (unsigned)__cvta_generic_to_shared(perm_tile + perm_swz((int)pos));
     }
+    dep_wait(src, dst);
     // origin of box o in source and destination, and the last index inside the
     // array along the cut axes
     auto origin = [&](unsigned o, unsigned& sb, unsigned& db, unsigned& lim) {
@@ -458,8 +460,7 @@ cudaError_t permute(const double* src, double* dst, int ndim, const int* dims, c
             g.dim[a] = dim[a];
             g.stride[a] = ss[a];
         }
-        ++g_launches;
-        k_permute_gather<<<(unsigned)((total + 255) / 256), 256, 0, s>>>(src, dst, (unsigned)total, g);
+        launch_dep(k_permute_gather, (unsigned)((total + 255) / 256), 256, 0, s, src, dst, (unsigned)total, g);
         return cudaGetLastError();
     }
     unsigned st = 1;
@@ -544,8 +545,7 @@ cudaError_t permute(const double* src, double* dst, int ndim, const int* dims, c
         const cudaError_t e = cudaFuncSetAttribute(k_permute, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (e != cudaSuccess) return e;
     }
-    ++g_launches;
-    k_permute<<<(unsigned)std::min<unsigned long long>(boxes, 152 * PERM_CTAS), PERM_THREADS, smem, s>>>(src, dst, p);
+    launch_dep(k_permute, (unsigned)std::min<unsigned long long>(boxes, 152 * PERM_CTAS), PERM_THREADS, smem, s, src, dst, p);
     return cudaGetLastError();
 }
 
@@ -554,6 +554,7 @@ cudaError_t permute(const double* src, double* dst, int ndim, const int* dims, c
 // ---------------------------------------------------------------------------
 namespace {
 __global__ void k_scale_cols(double* X, int rows, int cols, int ld, const double* __restrict__ w) {
+    dep_wait(X, w);
     const size_t total = (size_t)rows * cols;
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
         const int r = (int)(i / cols), c = (int)(i % cols);
@@ -561,6 +562,7 @@ __global__ void k_scale_cols(double* X, int rows, int cols, int ld, const double
     }
 }
 __global__ void k_inv_sqrt_cut(const double* __restrict__ sv, double* __restrict__ w, int n, double cut) {
+    dep_wait(sv, w);
     const double s0 = sv[0];
     for (int j = threadIdx.x; j < n; j += blockDim.x) {
         const double v = sv[j];
@@ -568,6 +570,7 @@ __global__ void k_inv_sqrt_cut(const double* __restrict__ sv, double* __restrict
     }
 }
 __global__ void k_maxabs(const double* __restrict__ x, size_t n, unsigned long long* maxbits) {
+    dep_wait(x, maxbits);
     double m = 0.0;
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
         const double a = fabs(x[i]);
@@ -593,6 +596,7 @@ __global__ void k_maxabs(const double* __restrict__ x, size_t n, unsigned long l
     }
 }
 __global__ void k_scale_by_max(double* x, size_t n, const unsigned long long* maxbits, int* flag) {
+    dep_wait(x, maxbits, flag);
     const unsigned long long b = *maxbits;
     if (b >= 0x7ff0000000000000ull) {  // Inf or NaN
         if (blockIdx.x == 0 && threadIdx.x == 0) atomicExch(flag, 1);
@@ -643,6 +647,7 @@ __global__ void k_rng_normal(double* __restrict__ out, size_t n, uint64_t seed, 
 constexpr int DOT_BLOCKS = 152 * 4;
 __global__ void k_dot_partial(const double* __restrict__ x, const double* __restrict__ y, size_t n,
                               double* __restrict__ part) {
+    dep_wait(x, y, part);
     double acc = 0.0;
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
         acc = fma(x[i], y[i], acc);
@@ -658,6 +663,7 @@ __global__ void k_dot_partial(const double* __restrict__ x, const double* __rest
     }
 }
 __global__ void k_dot_final(const double* __restrict__ part, int np, double* __restrict__ out) {
+    dep_wait(part, out);
     __shared__ double sm[256];
     double t = 0.0;
     for (int i = threadIdx.x; i < np; i += blockDim.x) t += part[i];
@@ -671,6 +677,7 @@ __global__ void k_dot_final(const double* __restrict__ part, int np, double* __r
 }
 // T[a,k,k',b] <- (T[a,k,k',b] + T[a,k',k,b]) / 2, one thread per pair k <= k'
 __global__ void k_sym_kk(double* __restrict__ T, int chi, int D) {
+    dep_wait(T);
     const size_t total = (size_t)chi * D * D * chi;
     for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < total; t += (size_t)gridDim.x * blockDim.x) {
         const size_t b = t % chi, kk2 = (t / chi) % D, kk = (t / ((size_t)chi * D)) % D, a = t / ((size_t)chi * D * D);
@@ -690,6 +697,7 @@ inline unsigned grid_for(size_t n, unsigned threads = 256) {
 // dst[i][j] += src[i][j] for a rows x cols block (row strides lds, ldd)
 __global__ void k_add_block(const double* __restrict__ src, int rows, int cols, int lds, double* __restrict__ dst,
                             int ldd) {
+    dep_wait(src, dst);
     const size_t total = (size_t)rows * cols;
     for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < total; t += (size_t)gridDim.x * blockDim.x) {
         const int i = (int)(t / cols), j = (int)(t % cols);
@@ -700,32 +708,27 @@ __global__ void k_add_block(const double* __restrict__ src, int rows, int cols, 
 
 cudaError_t add_block(const double* src, int rows, int cols, int lds, double* dst, int ldd, cudaStream_t s) {
     if (rows <= 0 || cols <= 0) return cudaSuccess;
-    ++g_launches;
-    k_add_block<<<grid_for((size_t)rows * cols), 256, 0, s>>>(src, rows, cols, lds, dst, ldd);
+    launch_dep(k_add_block, grid_for((size_t)rows * cols), 256, 0, s, src, rows, cols, lds, dst, ldd);
     return cudaGetLastError();
 }
 
 cudaError_t scale_cols(double* X, int rows, int cols, int ld, const double* w, cudaStream_t s) {
     if (rows <= 0 || cols <= 0) return cudaSuccess;
-    ++g_launches;
-    k_scale_cols<<<grid_for((size_t)rows * cols), 256, 0, s>>>(X, rows, cols, ld, w);
+    launch_dep(k_scale_cols, grid_for((size_t)rows * cols), 256, 0, s, X, rows, cols, ld, w);
     return cudaGetLastError();
 }
 cudaError_t inv_sqrt_cut(const double* sv, double* w, int n, double cut, cudaStream_t s) {
-    ++g_launches;
-    k_inv_sqrt_cut<<<1, 256, 0, s>>>(sv, w, n, cut);
+    launch_dep(k_inv_sqrt_cut, 1, 256, 0, s, sv, w, n, cut);
     return cudaGetLastError();
 }
 cudaError_t maxabs(const double* x, size_t n, unsigned long long* maxbits, cudaStream_t s) {
     if (!n) return cudaSuccess;
-    ++g_launches;
-    k_maxabs<<<grid_for(n), 256, 0, s>>>(x, n, maxbits);
+    launch_dep(k_maxabs, grid_for(n), 256, 0, s, x, n, maxbits);
     return cudaGetLastError();
 }
 cudaError_t scale_by_max(double* x, size_t n, const unsigned long long* maxbits, int* flag, cudaStream_t s) {
     if (!n) return cudaSuccess;
-    ++g_launches;
-    k_scale_by_max<<<grid_for(n), 256, 0, s>>>(x, n, maxbits, flag);
+    launch_dep(k_scale_by_max, grid_for(n), 256, 0, s, x, n, maxbits, flag);
     return cudaGetLastError();
 }
 // FP64 FMA throughput probe: every thread runs 8 independent FMA chains
@@ -746,6 +749,7 @@ __global__ void k_dfma_probe(double* __restrict__ out, int iters, double a, doub
 
 // out[m] = trace of the n x n matrix As + m n^2, m < nm (one warp per matrix)
 __global__ void k_traces(const double* __restrict__ As, int n, int nm, double* __restrict__ out) {
+    dep_wait(As, out);
     const int m = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (m >= nm) return;
     const double* a = As + (size_t)m * n * n;
@@ -757,15 +761,12 @@ __global__ void k_traces(const double* __restrict__ As, int n, int nm, double* _
 
 size_t dot_ws_doubles() { return DOT_BLOCKS; }
 cudaError_t dot(const double* x, const double* y, size_t n, double* out, double* ws, cudaStream_t s) {
-    ++g_launches;
-    k_dot_partial<<<DOT_BLOCKS, 256, 0, s>>>(x, y, n, ws);
-    ++g_launches;
-    k_dot_final<<<1, 256, 0, s>>>(ws, DOT_BLOCKS, out);
+    launch_dep(k_dot_partial, DOT_BLOCKS, 256, 0, s, x, y, n, ws);
+    launch_dep(k_dot_final, 1, 256, 0, s, ws, DOT_BLOCKS, out);
     return cudaGetLastError();
 }
 cudaError_t traces(const double* As, int n, int nm, double* out, cudaStream_t s) {
-    ++g_launches;
-    k_traces<<<(nm + 7) / 8, 256, 0, s>>>(As, n, nm, out);
+    launch_dep(k_traces, (nm + 7) / 8, 256, 0, s, As, n, nm, out);
     return cudaGetLastError();
 }
 cudaError_t dfma_probe(double* out, int blocks, int threads, int iters, cudaStream_t s) {
@@ -774,8 +775,7 @@ cudaError_t dfma_probe(double* out, int blocks, int threads, int iters, cudaStre
     return cudaGetLastError();
 }
 cudaError_t sym_kk(double* T, int chi, int D, cudaStream_t s) {
-    ++g_launches;
-    k_sym_kk<<<grid_for((size_t)chi * D * D * chi), 256, 0, s>>>(T, chi, D);
+    launch_dep(k_sym_kk, grid_for((size_t)chi * D * D * chi), 256, 0, s, T, chi, D);
     return cudaGetLastError();
 }
 cudaError_t rng_normal(double* out, size_t n, uint64_t seed, uint64_t sid, cudaStream_t s) {

@@ -348,6 +348,7 @@ __device__ __forceinline__ unsigned slice_of_pair(unsigned long long za, unsigne
 template <bool PLAIN>
 __global__ void __launch_bounds__(128) k_rowmax_cols(const double* __restrict__ X, int R, int K, View rv, View kv,
                                                      int kranges, int krange, unsigned long long* __restrict__ maxbits) {
+    dep_wait(X, maxbits);
     const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     const int rg = w / kranges, kr = w - rg * kranges;
     const int r = rg * 32 + lane;
@@ -421,6 +422,7 @@ __device__ __forceinline__ long long scaled_round(double x, int e, int nbits) {
 __global__ void k_split_tf32(const double* __restrict__ X, int R, int K, int K4, View rv, View kv,
                              const unsigned long long* __restrict__ maxbits, float* __restrict__ out,
                              int* __restrict__ ex) {
+    dep_wait(X, maxbits, out, ex);
     const long long tid = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     const int nq = K4 / 4;
     const long long r = tid / nq;
@@ -462,6 +464,7 @@ template <int TPR, bool VEC>
 __global__ void __launch_bounds__(256) k_split_rows_reg(const double* __restrict__ X, int R, int K, int K8,
                                                        long long rs, int s, __nv_bfloat16* __restrict__ out,
                                                        int* __restrict__ ex) {
+    dep_wait(X, out, ex);
     constexpr int RPB = 256 / TPR;
     __shared__ unsigned long long red[8];
     const int g = threadIdx.x / TPR, j = threadIdx.x % TPR;
@@ -537,6 +540,7 @@ __global__ void __launch_bounds__(256) k_split_rows_reg(const double* __restrict
 constexpr int ROWS_KRANGE = 1024;
 __global__ void __launch_bounds__(256) k_rowmax_rows(const double* __restrict__ X, int R, int K, View rv, View kv,
                                                     int kranges, unsigned long long* __restrict__ maxbits) {
+    dep_wait(X, maxbits);
     const long long w = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     const long long r = w / kranges;
@@ -553,6 +557,7 @@ __global__ void __launch_bounds__(256) k_split_rows_long(const double* __restric
                                                         View kv, int s,
                                                         const unsigned long long* __restrict__ maxbits,
                                                         __nv_bfloat16* __restrict__ out, int* __restrict__ ex) {
+    dep_wait(X, maxbits, out, ex);
     const int nch = K8 >> 3;
     const long long tid = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     const long long r = tid / nch;
@@ -639,6 +644,7 @@ __global__ void __launch_bounds__(64, 8) k_split_cols(const double* __restrict__
                                                   int s, const unsigned long long* __restrict__ maxbits,
                                                   __nv_bfloat16* __restrict__ out, int* __restrict__ ex, int kspan,
                                                   int kgroups) {
+    dep_wait(X, maxbits, out, ex);
     __shared__ uint4 tile[2][32][5];  // +1 uint4 per row against bank conflicts
     const int wid = (int)((blockIdx.x * (size_t)blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
     const int rg = wid / kgroups, kg = wid - rg * kgroups;
@@ -677,6 +683,7 @@ __global__ void __launch_bounds__(32 * COLS_ONE_WARPS) k_split_cols_one(const do
                                                                        View rv, View kv, int s,
                                                                        __nv_bfloat16* __restrict__ out,
                                                                        int* __restrict__ ex) {
+    dep_wait(X, out, ex);
     __shared__ uint4 tile[COLS_ONE_WARPS][32][5];
     __shared__ unsigned long long red[COLS_ONE_WARPS][32], all[16][32];  // of the warps; of the cluster's CTAs
     cg::cluster_group cl = cg::this_cluster();
@@ -1042,6 +1049,7 @@ __global__ void __launch_bounds__(THREADS, 1)
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
+    dep_wait();  // the operands and the outputs are touched from here on only
 
     if (warp == EPI_WARPS) {
         // ---------------- TMA producer ----------------
@@ -1319,6 +1327,7 @@ __global__ void __launch_bounds__(SHORT_THREADS, 1)
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
+    dep_wait();  // the operands and the outputs are touched from here on only
 
     if (warp == 2 * TEAM_WARPS) {
         // ---------------- TMA producer ----------------
@@ -1441,6 +1450,7 @@ constexpr int COMBINE_INT64_K = 1 << 17;
 __global__ void k_oz_combine(const long long* __restrict__ PZ, int splits, int wide, int Mpad, int Npad, int M, int N,
                              const int* __restrict__ eA, const int* __restrict__ eB, double alpha, double beta,
                              double* __restrict__ C, View out_r, View out_c) {
+    dep_wait(PZ, eA, eB, C);
     const size_t total = (size_t)M * N, zs = (size_t)Mpad * Npad;
     for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < total; t += (size_t)gridDim.x * blockDim.x) {
         const int m = (int)(t / N), n = (int)(t % N);
@@ -1608,9 +1618,7 @@ cudaError_t launch_gemm(GemmKernel kern, int threads, unsigned long long* done, 
         const long long tiles = (long long)p.m_tiles * p.n_tiles;
         grid = dim3((unsigned)std::min<long long>(tiles, nsm > 0 ? nsm : 1), 1, 1);
     }
-    ++g_launches;
-    kern<<<grid, threads, p.smem, st>>>(ta, tb, g);
-    return cudaGetLastError();
+    return launch_dep(kern, grid, threads, p.smem, st, ta, tb, g);
 }
 template <int NB16>
 cudaError_t launch_mode(int mode, const Plan& p, const CUtensorMap& ta, const CUtensorMap& tb, const oz::GemmArgs& g,
@@ -1704,8 +1712,8 @@ static int cols_cluster(int R, int K8) {
 
 static void launch_rowmax_cols(unsigned blocks, cudaStream_t st, const double* X, int R, int K, const oz::View& rv,
                                const oz::View& kv, int kranges, int krange, unsigned long long* mb) {
-    if (kv.n == 1) oz::k_rowmax_cols<true><<<blocks, 128, 0, st>>>(X, R, K, rv, kv, kranges, krange, mb);
-    else oz::k_rowmax_cols<false><<<blocks, 128, 0, st>>>(X, R, K, rv, kv, kranges, krange, mb);
+    launch_dep(kv.n == 1 ? oz::k_rowmax_cols<true> : oz::k_rowmax_cols<false>, blocks, 128, 0, st, X, R, K, rv, kv, kranges,
+               krange, mb);
 }
 
 cudaError_t oz_split_tf32(const double* X, int R, int K, const OzView& rvh, const OzView& kvh, void* buf,
@@ -1732,18 +1740,16 @@ cudaError_t oz_split_tf32(const double* X, int R, int K, const OzView& rvh, cons
     const unsigned long long warps = (unsigned long long)rg * kr;
     const unsigned long long threads = (unsigned long long)R * (K4 / 4);
     if ((warps + 3) / 4 > 0x7fffffffull || (threads + 255) / 256 > 0x7fffffffull) return cudaErrorInvalidValue;
-    ++g_launches;
     launch_rowmax_cols((unsigned)((warps + 3) / 4), st, X, R, K, rv, kv, (int)kr, krange, mb);
-    ++g_launches;
-    oz::k_split_tf32<<<(unsigned)((threads + 255) / 256), 256, 0, st>>>(X, R, K, K4, rv, kv, mb, sl, ex);
+    launch_dep(oz::k_split_tf32, (unsigned)((threads + 255) / 256), 256, 0, st, X, R, K, K4, rv, kv, mb, sl, ex);
     return cudaGetLastError();
 }
 
 template <int TPR>
 void launch_rows_reg_t(bool vec, unsigned blocks, cudaStream_t st, const double* X, int R, int K, int K8,
                        long long rs, int s, __nv_bfloat16* sl, int* ex) {
-    if (vec) oz::k_split_rows_reg<TPR, true><<<blocks, 256, 0, st>>>(X, R, K, K8, rs, s, sl, ex);
-    else oz::k_split_rows_reg<TPR, false><<<blocks, 256, 0, st>>>(X, R, K, K8, rs, s, sl, ex);
+    launch_dep(vec ? oz::k_split_rows_reg<TPR, true> : oz::k_split_rows_reg<TPR, false>, blocks, 256, 0, st, X, R, K, K8, rs,
+               s, sl, ex);
 }
 void launch_split_rows_reg(int tpr, bool vec, unsigned blocks, cudaStream_t st, const double* X, int R, int K,
                            int K8, long long rs, int s, __nv_bfloat16* sl, int* ex) {
@@ -1789,7 +1795,6 @@ cudaError_t oz_split_view(const double* X, int R, int K, const OzView& rvh, cons
         while (tpr * 4 < nch) tpr *= 2;
         const bool vec = ((uintptr_t)X % 16 == 0) && (rv.stride[0] % 2 == 0);
         const unsigned blocks = (unsigned)(((size_t)R * tpr + 255) / 256);
-        ++g_launches;
         launch_split_rows_reg(tpr, vec, blocks, st, X, R, K, K8, rv.stride[0], s, sl, ex);
     } else if (cs == 1) {
         cudaError_t e = cudaMemsetAsync(mb, 0, (size_t)R * 8, st);
@@ -1797,26 +1802,12 @@ cudaError_t oz_split_view(const double* X, int R, int K, const OzView& rvh, cons
         const int kr = (K + oz::ROWS_KRANGE - 1) / oz::ROWS_KRANGE;
         const unsigned long long b1 = ((unsigned long long)R * kr + 7) / 8, b2 = ((unsigned long long)R * nch + 255) / 256;
         if (b1 > 0x7fffffffull || b2 > 0x7fffffffull) return cudaErrorInvalidValue;
-        ++g_launches;
-        oz::k_rowmax_rows<<<(unsigned)b1, 256, 0, st>>>(X, R, K, rv, kv, kr, mb);
-        ++g_launches;
-        oz::k_split_rows_long<<<(unsigned)b2, 256, 0, st>>>(X, R, K, K8, rv, kv, s, mb, sl, ex);
+        launch_dep(oz::k_rowmax_rows, (unsigned)b1, 256, 0, st, X, R, K, rv, kv, kr, mb);
+        launch_dep(oz::k_split_rows_long, (unsigned)b2, 256, 0, st, X, R, K, K8, rv, kv, s, mb, sl, ex);
     } else if (const int nc = cols_cluster(R, K8)) {
         const int warps = std::min(oz::COLS_ONE_WARPS, ((K8 + 31) / 32 + nc - 1) / nc);
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3((unsigned)((R + 31) / 32 * nc), 1, 1);
-        cfg.blockDim = dim3((unsigned)(32 * warps), 1, 1);
-        cfg.stream = st;
-        cudaLaunchAttribute at[1];
-        at[0].id = cudaLaunchAttributeClusterDimension;
-        at[0].val.clusterDim.x = (unsigned)nc;
-        at[0].val.clusterDim.y = 1;
-        at[0].val.clusterDim.z = 1;
-        cfg.attrs = at;
-        cfg.numAttrs = 1;
-        ++g_launches;
-        return cudaLaunchKernelEx(&cfg, kv.n == 1 ? oz::k_split_cols_one<true> : oz::k_split_cols_one<false>, X, R, K, K8,
-                                  rv, kv, s, sl, ex);
+        return launch_dep_cluster(kv.n == 1 ? oz::k_split_cols_one<true> : oz::k_split_cols_one<false>, nc,
+                                  (unsigned)((R + 31) / 32 * nc), 32 * warps, 0, st, X, R, K, K8, rv, kv, s, sl, ex);
     } else {
         cudaError_t e = cudaMemsetAsync(mb, 0, (size_t)R * 8, st);
         if (e != cudaSuccess) return e;
@@ -1827,12 +1818,10 @@ cudaError_t oz_split_view(const double* X, int R, int K, const OzView& rvh, cons
         const int kspan = std::min(oz::COLS_SPAN, cols_krange(R, K8)), kgroups = (K8 + kspan - 1) / kspan;
         const unsigned long long warps2 = (unsigned long long)rg * kgroups;
         if ((warps + 3) / 4 > 0x7fffffffull || (warps2 + 1) / 2 > 0x7fffffffull) return cudaErrorInvalidValue;
-        ++g_launches;
         launch_rowmax_cols((unsigned)((warps + 3) / 4), st, X, R, K, rv, kv, (int)kr, krange, mb);
         const unsigned blocks = (unsigned)((warps2 + 1) / 2);
-        ++g_launches;
-        if (kv.n == 1) oz::k_split_cols<true><<<blocks, 64, 0, st>>>(X, R, K, K8, rv, kv, s, mb, sl, ex, kspan, kgroups);
-        else oz::k_split_cols<false><<<blocks, 64, 0, st>>>(X, R, K, K8, rv, kv, s, mb, sl, ex, kspan, kgroups);
+        launch_dep(kv.n == 1 ? oz::k_split_cols<true> : oz::k_split_cols<false>, blocks, 64, 0, st, X, R, K, K8, rv, kv, s, mb,
+                   sl, ex, kspan, kgroups);
     }
     return cudaGetLastError();
 }
@@ -1925,8 +1914,7 @@ cudaError_t oz_gemm_view(int M, int N, int K, int s, const void* Asplit, const v
     if (e != cudaSuccess || g.direct) return e;
     size_t blocks = ((size_t)M * N + 255) / 256;
     if (blocks > 152 * 16) blocks = 152 * 16;
-    ++g_launches;
-    oz::k_oz_combine<<<(unsigned)blocks, 256, 0, st>>>(g.PZ, p.ksplit, K > oz::COMBINE_INT64_K ? 1 : 0, g.Mpad, g.Npad,
+    launch_dep(oz::k_oz_combine, (unsigned)blocks, 256, 0, st, g.PZ, p.ksplit, K > oz::COMBINE_INT64_K ? 1 : 0, g.Mpad, g.Npad,
                                                         M, N, g.eA, g.eB, alpha, beta, C, g.out_r, g.out_c);
     return cudaGetLastError();
 }
