@@ -929,7 +929,13 @@ ctm_status one_sweep(ctm_ctx* h) {
     if (!h->use_graphs || h->prof || !steady) return one_sweep_eager(h);
     if (!h->graph_exec) {
         CK(cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal));
-        const ctm_status st = one_sweep_eager(h);
+        const ctm_status st = [&] {
+            struct Own {
+                Own() { ctm::dep_in_capture = true; }
+                ~Own() { ctm::dep_in_capture = false; }
+            } own;
+            return one_sweep_eager(h);
+        }();
         cudaGraph_t g = nullptr;
         const cudaError_t e = cudaStreamEndCapture(h->stream, &g);
         if (st != CTM_OK) {

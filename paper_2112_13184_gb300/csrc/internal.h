@@ -20,11 +20,14 @@ extern std::atomic<long long> g_launches;
 // dep_wait until its writes are visible: every such kernel calls dep_wait in
 // every thread before it touches global memory.  Chains of kernels of a few
 // microseconds are bound by the gaps in between: correlations at d=2, D=5,
-// chi=48 (3000 launches) 36.6 -> 29.7 ms, the scan point at D=4, chi=32 16.9 -> 15.3.
+// chi=48 (3000 launches) 36.6 -> 29.3 ms, the scan point at D=4, chi=32 16.9 -> 14.8.
 // No kernel lets its successor in before it ends: with that, waiting blocks
 // held the places of running ones (the same correlations 32.1 ms, the density
 // matrices at d=3, D=8, chi=64 56.8 ms against 53.0).
-// A capturing stream gets plain launches, so that a graph has plain edges.
+// A capturing stream gets plain launches, so that a caller's graph has plain
+// edges; a handle's own sweep graph (dep_in_capture, set by the thread that
+// captures it for as long as that takes) has programmatic ones.
+extern thread_local bool dep_in_capture;
 template <class... KA, class... A>
 cudaError_t launch_dep_cluster(void (*kernel)(KA...), int cluster, dim3 grid, dim3 block, size_t smem, cudaStream_t s,
                                A... a) {
@@ -43,7 +46,7 @@ cudaError_t launch_dep_cluster(void (*kernel)(KA...), int cluster, dim3 grid, di
     }
     cfg.attrs = at;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusActive;
-    if (cudaStreamIsCapturing(s, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone) {
+    if (dep_in_capture || (cudaStreamIsCapturing(s, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone)) {
         at[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
         at[cfg.numAttrs].val.programmaticStreamSerializationAllowed = 1;
         ++cfg.numAttrs;

@@ -10,6 +10,7 @@
 namespace ctm {
 
 std::atomic<long long> g_launches{0};
+thread_local bool dep_in_capture = false;
 
 // ---------------------------------------------------------------------------
 // FP64 GEMM, row-major: C[M,N] = alpha op(A) op(B) + beta C.
