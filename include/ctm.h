@@ -112,8 +112,12 @@ typedef struct {
     int batch_cuts;         /* != 0: the two row cuts of a column step are processed
                                together -- both cuts' enlarged corners stay
                                resident (4 N^2 more doubles and, in a tensor-core
-                               mode, 8 more slice caches) and their projector
-                               SVDs run in one launch                          */
+                               mode, 8 more slice caches), their projector
+                               SVDs run in one launch, and corners that the next
+                               cut needs again are kept instead of computed
+                               twice; where one cut leaves the chip idle the two
+                               run side by side, the second on a stream of the
+                               handle's own, joined before the call's work ends */
 } ctm_options;
 
 /* Defaults: chi=16, max_sweeps=100, tol=1e-10, FP64, 5 slices,
@@ -340,10 +344,12 @@ ctm_status ctm_permute(const double* src, double* dst, int ndim, const int* dims
 /* Thin Householder QR of Y (N x k row-major, N >= k): Q (N x k) with
  * orthonormal columns and upper-triangular R (k x k, diagonal >= 0), Y=QR.
  * Y is not modified.  ws: workspace of ctm_qr_workspace_bytes(N,k) bytes.
- * Runs as one persistent cooperative launch over all SMs when the row slabs
- * fit in shared memory (k columns of ~N/152 rows twice), else as two
- * launches per column; in the persistent form the first int of ws is set to
- * 1 if a bounded grid barrier gave up (Q and R then hold no result). */
+ * Runs as one blocked launch when the row slabs fit in shared memory (k
+ * columns of N divided by the blocks): a cluster of up to 16 blocks where
+ * exchanges weigh more than arithmetic (small N k), else a cooperative
+ * launch over the SMs; without either as two launches per column.  In the
+ * cooperative form the first int of ws is set to 1 if a bounded grid barrier
+ * gave up (Q and R then hold no result). */
 size_t ctm_qr_workspace_bytes(int N, int k);
 ctm_status ctm_qr(const double* Y, int N, int k, double* Q, double* R, void* ws, void* stream);
 
