@@ -5,6 +5,7 @@
 #include <cmath>
 #include <cstdint>
 
+#include "dgemm_plan.h"
 #include "internal.h"
 
 namespace ctm {
@@ -25,9 +26,6 @@ thread_local bool dep_in_capture = false;
 // its products) 293 -> 146 ms, at d=2, D=3, chi=16 51 -> 6.5 ms.
 // ---------------------------------------------------------------------------
 namespace {
-constexpr int GK = 16;
-constexpr int GMAX_TM = 4, GMAX_TN = 9;
-
 // Split-K: blockIdx.z takes K range [z*kchunk, (z+1)*kchunk) and writes its
 // partial product (alpha=1, beta=0) to C + z*zstride; a second kernel sums
 // the partials in fixed order, so results do not depend on scheduling.
@@ -42,8 +40,9 @@ __global__ void __launch_bounds__(256) k_dgemm(int M, int N, int K, double alpha
     constexpr int NA = BM * GK / 256, NB = (BN * GK + 255) / 256;
     __shared__ double As[GK][BM + 1];
     __shared__ double Bs[GK][BN + 1];
-    const int kbeg = blockIdx.z * kchunk;
-    const int kend = min(K, kbeg + kchunk);
+    // unsigned: the ends of the last split and step may lie beyond 2^31
+    const unsigned kbeg = blockIdx.z * (unsigned)kchunk;
+    const unsigned kend = min((unsigned)K, kbeg + (unsigned)kchunk);
     C += blockIdx.z * zstride;
     const int tid = threadIdx.x, tx = tid & 7, ty = tid >> 3;
     const long long m0 = (long long)blockIdx.x * BM, n0 = (long long)blockIdx.y * BN;
@@ -55,7 +54,7 @@ __global__ void __launch_bounds__(256) k_dgemm(int M, int N, int K, double alpha
 #pragma unroll
         for (int j = 0; j < TN; ++j) acc[i][j] = 0.0;
     double pa[NA], pb[NB];
-    auto load = [&](int k0) {
+    auto load = [&](unsigned k0) {
 #pragma unroll
         for (int r = 0; r < NA; ++r) {
             const int idx = tid + 256 * r;
@@ -72,7 +71,7 @@ __global__ void __launch_bounds__(256) k_dgemm(int M, int N, int K, double alpha
         }
     };
     if (kbeg < kend) load(kbeg);
-    for (int k0 = kbeg; k0 < kend; k0 += GK) {
+    for (unsigned k0 = kbeg; k0 < kend; k0 += GK) {
         __syncthreads();
 #pragma unroll
         for (int r = 0; r < NA; ++r) {
@@ -88,7 +87,7 @@ __global__ void __launch_bounds__(256) k_dgemm(int M, int N, int K, double alpha
         }
         __syncthreads();
         if (k0 + GK < kend) load(k0 + GK);
-        const int nk = min(GK, kend - k0);
+        const int nk = (int)min((unsigned)GK, kend - k0);
         for (int kk = 0; kk < nk; ++kk) {
             double a[TM], b[TN];
 #pragma unroll
@@ -180,40 +179,6 @@ __global__ void k_gemv_sum(const double* __restrict__ P, int parts, int M, doubl
     }
 }
 
-struct GemmPlan {
-    int tm = 1, tn = 1, splits = 1, kchunk = 1;
-};
-// The tile and K split with the least work on the fullest SM: TM TN multiply-
-// adds per thread and k, at ~150 cycles each (8 warps on 4 quarters, measured
-// 153), an estimated 3000 cycles of launch, fill and drain per CTA, 600 per 16
-// of K for loads that a small tile does not cover, and for a split its
-// partials' pass.
-GemmPlan dgemm_plan(int M, int N, int K, size_t ws_doubles) {
-    GemmPlan best;
-    double best_cost = -1.0;
-    for (int tm = 1; tm <= GMAX_TM; tm *= 2)
-        for (int tn = 1; tn <= GMAX_TN; ++tn) {
-            const double tiles = std::ceil(M / (32.0 * tm)) * std::ceil(N / (8.0 * tn));
-            if (tn < GMAX_TN && N > 8 * tn * 65535) continue;  // grid.y
-            for (int sp = 1; sp <= 256; sp *= 2) {
-                const int kc = ((K + sp - 1) / sp + GK - 1) / GK * GK;
-                const int s = (K + kc - 1) / kc;
-                if (sp > 1 && (s != sp || (size_t)s * M * N > ws_doubles)) break;
-                const double steps = std::ceil(kc / (double)GK), per = (double)tm * tn * std::min(kc, K) * 150.0;
-                const double cta = std::max(per, 600.0 * steps) + 300.0 * steps + 3000.0;
-                const double cost = std::ceil(tiles * s / 152.0) * cta + (s > 1 ? 6000.0 + 40.0 * s * M * N / 152.0 / 32.0 : 0.0);
-                if (best_cost < 0.0 || cost < best_cost) {
-                    best_cost = cost;
-                    best.tm = tm;
-                    best.tn = tn;
-                    best.splits = s;
-                    best.kchunk = kc;
-                }
-            }
-        }
-    return best;
-}
-
 struct GemmArgs64 {
     int M, N, K;
     double alpha;
@@ -251,6 +216,7 @@ cudaError_t dgemm(bool tA, bool tB, int M, int N, int K, double alpha, const dou
                   const double* B, int ldb, double beta, double* C, int ldc, cudaStream_t s, double* ws,
                   size_t ws_doubles) {
     if (M <= 0 || N <= 0) return cudaSuccess;
+    if (N > DGEMM_MAX_N) return cudaErrorInvalidValue;
     if (N == 1 && !tA && M <= GEMV_ROWS && K >= (1 << 16) && ws && ws_doubles >= (size_t)GEMV_CTAS * M) {
         launch_dep(k_gemv_long, GEMV_CTAS, 256, 0, s, M, K, A, lda, B, tB ? 1 : ldb, ws);
         launch_dep(k_gemv_sum, 1, 32 * M, 0, s, ws, GEMV_CTAS, M, alpha, beta, C, ldc);
@@ -259,7 +225,6 @@ cudaError_t dgemm(bool tA, bool tB, int M, int N, int K, double alpha, const dou
     const GemmPlan p = dgemm_plan(M, N, K, ws ? ws_doubles : 0);
     const dim3 grid((unsigned)((M + 32 * p.tm - 1) / (32 * p.tm)), (unsigned)((N + 8 * p.tn - 1) / (8 * p.tn)),
                     (unsigned)p.splits);
-    if (grid.y > 65535u) return cudaErrorInvalidValue;
     GemmArgs64 a{M, N, K, alpha, A, tA ? 1 : lda, tA ? lda : 1, B, tB ? 1 : ldb, tB ? ldb : 1, beta, C, ldc,
                  p.splits > 1 ? p.kchunk : std::max(K, 1), (size_t)M * N};
     if (p.splits > 1) {
