@@ -4,6 +4,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstdint>
+#include <mutex>
 
 #include "dgemm_plan.h"
 #include "internal.h"
@@ -387,6 +388,25 @@ k_permute(const double* __restrict__ src, double* __restrict__ dst, const __grid
     }
     asm volatile("cp.async.wait_group 0;" ::: "memory");
 }
+
+// The limit of k_permute's shared memory, for its largest box: an attribute of
+// the function on a device, not of a launch or a host thread, so it is set
+// once for each device.  (Set to every call's own size, another thread's call
+// could lower it between this one's setting and its launch.)
+cudaError_t permute_attributes() {
+    static std::mutex mu;
+    static unsigned long long done = 0;  // a bit per device
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+    std::lock_guard<std::mutex> lock(mu);
+    if (done >> dev & 1ull) return cudaSuccess;
+    constexpr int most = PERM_STAGES * (perm_swz(PERM_BOX - 1) + 1) * (int)sizeof(double);
+    e = cudaFuncSetAttribute(k_permute, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+    if (e == cudaSuccess) done |= 1ull << dev;
+    return e;
+}
 }  // namespace
 
 cudaError_t permute(const double* src, double* dst, int ndim, const int* dims, const int* perm,
@@ -507,10 +527,8 @@ cudaError_t permute(const double* src, double* dst, int ndim, const int* dims, c
     }
     p.boxes = (unsigned)boxes;
     const int smem = PERM_STAGES * p.tile * (int)sizeof(double);
-    if (smem > 48 * 1024) {
-        const cudaError_t e = cudaFuncSetAttribute(k_permute, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        if (e != cudaSuccess) return e;
-    }
+    const cudaError_t e = permute_attributes();
+    if (e != cudaSuccess) return e;
     launch_dep(k_permute, (unsigned)std::min<unsigned long long>(boxes, 152 * PERM_CTAS), PERM_THREADS, smem, s, src, dst, p);
     return cudaGetLastError();
 }
