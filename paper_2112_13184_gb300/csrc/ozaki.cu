@@ -1881,6 +1881,19 @@ cudaError_t oz_gemm_view(int M, int N, int K, int s, const void* Asplit, const v
     // columns must be contiguous and aligned for every row.
     g.w = oz::Weights{1 << 20, 1 << 22, 1 << 28, 1};
     g.plain = alpha == 1.0 && beta == 0.0;
+    // The exact-level epilogue holds a column's offset in 32 bits (in 64 it spilled:
+    // 262144 x 192 x 64 227 -> 241 us): views with a negative or longer one are
+    // refused, unless the product goes by the split partials.  No caller has one:
+    // the outputs of a handle that fits the device end far below 2^32 elements.
+    if (mode == 0 && g.direct) {
+        unsigned long long last = 0;
+        for (int a = 0; a < ocv.n; ++a) {
+            if (ocv.dim[a] < 2) continue;
+            if (ocv.stride[a] < 0 || ocv.stride[a] >= (1ll << 32)) return cudaErrorInvalidValue;
+            last += (unsigned long long)(ocv.dim[a] - 1) * (unsigned long long)ocv.stride[a];
+            if (last >= (1ull << 32)) return cudaErrorInvalidValue;
+        }
+    }
     g.vec = 1;
     if (g.plain)
         for (int v : {4, 2}) {
