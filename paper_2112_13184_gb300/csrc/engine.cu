@@ -717,7 +717,7 @@ ctm_status projectors(ctm_ctx* h, int slot, int cut) {
 
 // While it lives, the handle's calls go to the second branch's stream with
 // its scratch: opened after what the branch needs is enqueued on the handle's
-// stream, and followed by join_branch before anything that needs its results.
+// stream, and joined (both_cuts) before anything that needs its results.
 struct BranchScope {
     ctm_ctx* h;
     explicit BranchScope(ctm_ctx* h_) : h(h_) { exchange(); }
@@ -790,9 +790,10 @@ ctm_status svd2_(ctm_ctx* h, const CutBufs& a, const CutBufs& b) {
 // T_{m+3} of the next column's sites only, so its right-hand corners (c = m+1,
 // m+2, of all four sites after its two steps) stay what they are: the next
 // move takes the former as its upper-left corners (in its first step, before
-// it rewrites them) and the latter as its upper-right ones.  46 of a sweep's
-// 64 corners are computed; at most eight are kept beside the four of a step
-// that are new.
+// it rewrites them) and the latter as its upper-right ones.  Of a sweep's 64
+// corners 37 are computed, 40 where the cuts fork (both absorptions then take
+// a corner's buffer); at most eight are kept beside the four of a step that
+// are new.
 int corner_id(int site, int c) { return 4 * site + (c & 3); }
 // E[r], r < 8, for the corners ids[r]: resident ones by pointer, the others
 // computed into buffers that hold none of `keep` (a predicate) or of ids

@@ -20,7 +20,7 @@ extern std::atomic<long long> g_launches;
 // dep_wait until its writes are visible: every such kernel calls dep_wait in
 // every thread before it touches global memory.  Chains of kernels of a few
 // microseconds are bound by the gaps in between: correlations at d=2, D=5,
-// chi=48 (3000 launches) 36.6 -> 29.3 ms, the scan point at D=4, chi=32 16.9 -> 14.8.
+// chi=48 (3000 launches) 36.0 -> 29.5 ms, the scan point at D=4, chi=32 16.9 -> 15.3.
 // No kernel lets its successor in before it ends: with that, waiting blocks
 // held the places of running ones (the same correlations 32.1 ms, the density
 // matrices at d=3, D=8, chi=64 56.8 ms against 53.0).

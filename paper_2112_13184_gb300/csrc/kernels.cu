@@ -133,7 +133,8 @@ __global__ void k_splitk_reduce(const double* __restrict__ P, int splits, int M,
 // rows of chi^2 D^4): bound by reading A once.  Every CTA takes a K range and
 // all rows; the partials [CTA][row] are summed by one warp per row in fixed
 // order.  At d=3, D=8, chi=128 (9 x 1 x 67M; one 64 x 64 tile split 304 ways
-// before) the one-site density matrix went from 463 to 23 ms.  Shorter K, and
+// before) the one-site density matrix went from 463 to 23 ms, and to 11 with its
+// permutes by boxes.  Shorter K, and
 // calls without a workspace, stay with the tiles.
 constexpr int GEMV_ROWS = 16;
 constexpr int GEMV_CTAS = 152 * 4;

@@ -9,15 +9,14 @@
 // on the tensor cores in FP32 over K-chunks of 256 and read out of TMEM
 // after every chunk:
 //   level 0 (t+u = 0) and level 1 (t+u = 1) are integer-valued (in units of
-//   1 and 2^-8); over one chunk they stay below 2^24 units and are exact,
-//   and are added to int32 registers;
+//   1 and 2^-8); over one chunk they stay below 2^24 units and are exact;
 //   all pairs with 2 <= t+u <= s-1 carry a weight <= 2^-16 and share one
 //   FP32 accumulator, restarted every chunk so that the tensor cores'
-//   rounding does not grow with the magnitude accumulated over K; the chunk
-//   values are added in an FP32 register;
+//   rounding does not grow with the magnitude accumulated over K;
 //   pairs with t+u >= s are dropped (same order as the slicing error).
-// The result is assembled exactly in int64, C = 2^(eA+eB-16) (S0 + 2^-8 S1
-// + F).  Error: the slicing, 2^(2-8s) max|row| max|col| K, plus the tensor
+// Every chunk's S0 (level 0), S1 (level 1) and F (the rest) are added to one
+// int64 per entry, Z = 2^28 S0 + 2^20 S1 + round(2^28 F), and C = 2^(eA+eB-44)
+// Z.  Error: the slicing, 2^(2-8s) max|row| max|col| K, plus the tensor
 // cores' FP32 rounding of the levels >= 2 within a chunk, measured at about
 // 2^-36 max|row| max|col| K; so 5 slices reach ~1e-11 relative per unit K
 // and a 6th adds nothing.  Split-BF16 accumulated in FP32 over all of K
@@ -396,7 +395,7 @@ __global__ void __launch_bounds__(128) k_rowmax_cols(const double* __restrict__ 
 }
 
 // round(x 2^(nbits - e)) as an integer, |x| <= 2^e (integer operations on the
-// FP64 bit pattern, like digits())
+// FP64 bit pattern, as in digit_bytes)
 __device__ __forceinline__ long long scaled_round(double x, int e, int nbits) {
     const unsigned long long b = (unsigned long long)__double_as_longlong(x);
     int ex = (int)((b >> 52) & 0x7ff);
@@ -1648,8 +1647,6 @@ inline const int* split_tf32_exponents(const void* buf, int R, int K4) {
     return (const int*)((const char*)buf + align256((size_t)2 * R * K4 * 4) + align256((size_t)R * 8));
 }
 
-// K range of one warp in the lane = row kernels: 256, halved down to 32 until
-// the operand gives every SM sixteen warps
 // Whether the device runs clusters of 16 CTAs of the one-launch slicer (a
 // property of the device: asked once for each).
 static bool cols_cluster_of_16() {
@@ -1681,6 +1678,8 @@ static bool cols_cluster_of_16() {
     return ok;
 }
 
+// K range of one warp in the lane = row kernels: 256, halved down to 32 until
+// the operand gives every SM sixteen warps
 static int cols_krange(int R, int K) {
     const long long rg = (R + 31) / 32;
     int range = 256;
